@@ -498,14 +498,10 @@ sevennet_status ws_reserve(sevennet_model* M, Workspace* ws, int64_t n_atoms, in
         SN_TRY(ws_alloc(ws, &ws->row_ptr, N + 1));
         SN_TRY(ws_alloc(ws, &ws->row_cnt, N + 1));
         SN_TRY(ws_alloc(ws, &ws->pair_ptr, N + 1));
-        SN_TRY(ws_alloc(ws, &ws->h, N * M->h_max));
+        SN_TRY(ws_alloc(ws, &ws->quad_ptr, N + 1));
         SN_TRY(ws_alloc(ws, &ws->xs, (int64_t)T * N * M->x_max));
         SN_TRY(ws_alloc(ws, &ws->ys, (int64_t)T * N * M->y_max));
         SN_TRY(ws_alloc(ws, &ws->m, N * M->m_max));
-        SN_TRY(ws_alloc(ws, &ws->gy, N * M->y_max));
-        SN_TRY(ws_alloc(ws, &ws->gx, N * M->x_max));
-        SN_TRY(ws_alloc(ws, &ws->gxq, N * M->x_max));
-        SN_TRY(ws_alloc(ws, &ws->gh, N * M->h_max));
         SN_TRY(ws_alloc(ws, &ws->e_atom, N));
         SN_TRY(ws_alloc(ws, &ws->w_atom, N * 9));
         SN_TRY(ws_alloc(ws, &ws->f_s, N * 3));
@@ -525,6 +521,25 @@ sevennet_status ws_reserve(sevennet_model* M, Workspace* ws, int64_t n_atoms, in
         SN_TRY(ws_alloc(ws, &ws->p_geom, E));
         SN_TRY(ws_alloc(ws, &ws->gd, E * 3));
         ws->cap_edges = E;
+    }
+    const int64_t grad = std::max<int64_t>(ws->cap_atoms * st_grad_bytes(M), (ws->cap_edges + 1) / 2 * M->h2_bytes);
+    if (grad > ws->grad_bytes) {
+        ws->grad_bytes = 0;
+        SN_TRY(ws_alloc(ws, &ws->grad, grad));
+        ws->grad_bytes = grad;
+    }
+    if (M->h2_bytes && ws->cap_edges / 4 + ws->cap_atoms > ws->cap_quads) {
+        ws->cap_quads = 0;
+        SN_TRY(ws_alloc(ws, &ws->quads, ws->cap_edges / 4 + ws->cap_atoms));
+        ws->cap_quads = ws->cap_edges / 4 + ws->cap_atoms;
+    }
+    {
+        const int64_t N = ws->cap_atoms;
+        ws->gxq = reinterpret_cast<unsigned long long*>(ws->grad);
+        ws->gx = reinterpret_cast<float*>(ws->gxq + N * M->x_max);
+        ws->gy = ws->gx + N * M->x_max;
+        ws->gh = ws->gy + N * M->y_max;
+        ws->h = ws->gh + N * M->h_max;
     }
     if (n_bins + 1 > ws->cap_bins) {
         const int64_t B = std::max<int64_t>(n_bins + 1, 64);
@@ -572,8 +587,10 @@ void model_embed(sevennet_model* M, Workspace* ws, int64_t N, cudaStream_t st) {
 
 // Block t forward on all N atoms: x = Lin1(h), y = LinSC(h); m = conv(x);
 // y += Lin2(m); h = Gate(y).  x and y are kept for the adjoint.
+// pairs: the list is symmetric and its pairs are built (ws->pair_ptr, p_*, and the
+// pair of every edge in ws->gd): the streaming convolution runs where the model allows it.
 void model_layer_forward(sevennet_model* M, Workspace* ws, int t, int64_t N, int64_t E,
-                         sevennet_precision prec, cudaStream_t st) {
+                         sevennet_precision prec, cudaStream_t st, bool pairs) {
     const LayerDev& L = M->layers[t];
     Profiler* P = &M->prof;
     cudaEvent_t ev;
@@ -590,9 +607,17 @@ void model_layer_forward(sevennet_model* M, Workspace* ws, int t, int64_t N, int
     }
     run_gemm(M, g, prec, st);
     prof_begin(P, PF_CONV_FWD, st, &ev);
-    launch_conv_fwd(L, M->H, prec, N, E, ws->row_ptr, ws->dst, ws->src, ws->geom, x, ws->m, st, ws->flags);
-    prof_end(P, PF_CONV_FWD, st, ev, 1);
-    count_launches(1);
+    const bool stream = pairs && M->h2_bytes >= (prec == SEVENNET_BF16 ? 128 : 256);
+    if (stream) {
+        const int64_t cap = (ws->cap_edges + 1) / 2;
+        launch_radial(L, prec, cap, ws->pair_ptr + N, ws->p_geom, ws->grad, st);
+        launch_conv_fwd_stream(L, prec, N, cap, ws->row_ptr, ws->quad_ptr, ws->quads, ws->src, ws->geom,
+                               reinterpret_cast<const int*>(ws->gd), ws->grad, x, ws->m, ws->flags, st);
+    } else {
+        launch_conv_fwd(L, M->H, prec, N, E, ws->row_ptr, ws->dst, ws->src, ws->geom, x, ws->m, st, ws->flags);
+    }
+    prof_end(P, PF_CONV_FWD, st, ev, stream ? 2 : 1);
+    count_launches(stream ? 2 : 1);
     GemmBatch g2{};
     for (int l = 0; l < NL; ++l) {
         if (!L.y_mul[l] || !L.msg_mul[l]) continue;
@@ -675,17 +700,24 @@ sevennet_status run_model(sevennet_model* M, Workspace* ws, const BatchHost& b, 
     const int64_t N = b.atom_off[b.n_structs];
     const int T = M->T;
     cudaEvent_t ev;
+    // unordered pairs of the (symmetric) neighbour list, and the pair of every edge (kept in
+    // the memory of dE/dd, which the adjoint clears)
+    prof_begin(&M->prof, PF_NEIGHBORS, st, &ev);
+    build_pairs(ws, N, st);
+    if (M->h2_bytes) {
+        launch_pair_of((ws->cap_edges + 1) / 2, N, ws->row_ptr, ws->rev, ws->pair_ptr, ws->p_e,
+                       reinterpret_cast<int*>(ws->gd), st);
+        launch_quads(N, ws->row_ptr, ws->quad_ptr, ws->quads, st);
+    }
+    const int n_pre = M->h2_bytes ? 5 : 3;
+    prof_end(&M->prof, PF_NEIGHBORS, st, ev, n_pre);
+    count_launches(n_pre);
     model_embed(M, ws, N, st);
-    for (int t = 0; t < T; ++t) model_layer_forward(M, ws, t, N, E, prec, st);
+    for (int t = 0; t < T; ++t) model_layer_forward(M, ws, t, N, E, prec, st, true);
     model_readout(M, ws, N, st);
     // reverse path (E < 0: the edge count is on the device; clear the capacity)
     const int64_t E_clear = E < 0 ? ws->cap_edges : E;
     if (E_clear > 0) SN_CUDA(cudaMemsetAsync(ws->gd, 0, (size_t)E_clear * 3 * sizeof(float), st));
-    // the adjoint runs over unordered pairs of the (symmetric) neighbour list
-    prof_begin(&M->prof, PF_NEIGHBORS, st, &ev);
-    build_pairs(ws, N, st);
-    prof_end(&M->prof, PF_NEIGHBORS, st, ev, 3);
-    count_launches(3);
     for (int t = T - 1; t >= 0; --t) {
         model_layer_backward_gate(M, ws, t, N, st);
         SN_TRY(model_layer_backward_rest(M, ws, t, N, E, prec, st, true));
@@ -930,10 +962,14 @@ sevennet_status sevennet_create_model(const sevennet_model_config* cfg, const do
             if ((s = dev_upload(M, w2T, &L.mlp2T))) return fail(s);
             if ((s = dev_upload(M, to_bf16(w2T), &L.mlp2h))) return fail(s);   // [W][H]
             if ((s = dev_upload(M, to_bf16(w2), &L.mlp2Th))) return fail(s);   // [H][W]
+            if ((s = radial_pack(M, L))) return fail(s);
+            if ((s = st_plan_build(M, L))) return fail(s);
         }
     }
     sevennet_status s = conv_configure(H, M->layers);
+    if (!s) s = st_configure(M->lmax);
     if (s) return fail(s);
+    M->h2_bytes = st_h2_bytes(M);
     if (cudaStreamCreateWithFlags(&M->stream, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
         set_error("cudaStreamCreate failed");

@@ -119,6 +119,33 @@ __device__ __forceinline__ void envelope(const ConvDesc& D, float xr, float& u, 
     du = -D.env_a * p * xp1 + D.env_b * (p + 1.0f) * xp - D.env_c * (p + 2.0f) * xp2;
 }
 
+// Real harmonics of degree 1..LMAX of the unit vector (x, y, z), component
+// normalised, m = -l..l: Y[0..2] degree 1, Y[3..7] degree 2, Y[8..14] degree 3.
+template <int LMAX>
+__device__ __forceinline__ void edge_harmonics(float x, float y, float z, float* Y) {
+    const float s3 = 1.7320508075688772f, s15 = 3.872983346207417f, s5 = 2.23606797749979f;
+    Y[0] = s3 * y; Y[1] = s3 * z; Y[2] = s3 * x;
+    if constexpr (LMAX >= 2) {
+        Y[3] = s15 * x * y;
+        Y[4] = s15 * y * z;
+        Y[5] = 0.5f * s5 * (3.0f * z * z - 1.0f);
+        Y[6] = s15 * x * z;
+        Y[7] = 0.5f * s15 * (x * x - y * y);
+    }
+    if constexpr (LMAX >= 3) {   // degree 3: the standard real harmonics times sqrt(4 pi)
+        const float a3 = 2.0916500663351889f, b3 = 10.246950765959598f;    // sqrt(70)/4, sqrt(105)
+        const float c3 = 1.6201851746019651f, d3 = 1.3228756555322954f;    // sqrt(42)/4, sqrt(7)/2
+        const float zz5 = 5.0f * z * z;
+        Y[8] = a3 * y * (3.0f * x * x - y * y);
+        Y[9] = b3 * x * y * z;
+        Y[10] = c3 * y * (zz5 - 1.0f);
+        Y[11] = d3 * z * (zz5 - 3.0f);
+        Y[12] = c3 * x * (zz5 - 1.0f);
+        Y[13] = 0.5f * b3 * z * (x * x - y * y);
+        Y[14] = a3 * x * (x * x - 3.0f * y * y);
+    }
+}
+
 // Phase A: Y_l(d/r) (component normalised, m = -l..l) and the enveloped basis.
 template <int LMAX>
 __device__ __forceinline__ void edge_features(const ConvDesc& D, float4 g, float* Y, float* Bcol,
@@ -126,30 +153,9 @@ __device__ __forceinline__ void edge_features(const ConvDesc& D, float4 g, float
     const float r = g.w;
     const float inv = 1.0f / r;
     const float x = g.x * inv, y = g.y * inv, z = g.z * inv;
-    const float s3 = 1.7320508075688772f, s15 = 3.872983346207417f, s5 = 2.23606797749979f;
     Y[0] = 1.0f;
-    Y[1] = s3 * y; Y[2] = s3 * z; Y[3] = s3 * x;
-    if (D.lmax >= 2) {
-        Y[4] = s15 * x * y;
-        Y[5] = s15 * y * z;
-        Y[6] = 0.5f * s5 * (3.0f * z * z - 1.0f);
-        Y[7] = s15 * x * z;
-        Y[8] = 0.5f * s15 * (x * x - y * y);
-    } else {
-        Y[4] = Y[5] = Y[6] = Y[7] = Y[8] = 0.0f;
-    }
-    if constexpr (LMAX >= 3) {   // degree 3 (m = -3..3), the standard real harmonics times sqrt(4 pi)
-        const float a3 = 2.0916500663351889f, b3 = 10.246950765959598f;    // sqrt(70)/4, sqrt(105)
-        const float c3 = 1.6201851746019651f, d3 = 1.3228756555322954f;    // sqrt(42)/4, sqrt(7)/2
-        const float zz5 = 5.0f * z * z;
-        Y[9] = a3 * y * (3.0f * x * x - y * y);
-        Y[10] = b3 * x * y * z;
-        Y[11] = c3 * y * (zz5 - 1.0f);
-        Y[12] = d3 * z * (zz5 - 3.0f);
-        Y[13] = c3 * x * (zz5 - 1.0f);
-        Y[14] = 0.5f * b3 * z * (x * x - y * y);
-        Y[15] = a3 * x * (x * x - 3.0f * y * y);
-    }
+    edge_harmonics<LMAX>(x, y, z, Y + 1);
+    if constexpr (LMAX < 2) Y[4] = Y[5] = Y[6] = Y[7] = Y[8] = 0.0f;
     float u, du;
     envelope(D, r / D.r_cut, u, du);
     const float th = 3.14159265358979f * r / D.r_cut;

@@ -19,6 +19,7 @@
 // fragments of every path built from Y, the hidden MLP layer and w^T = W3^T H2^T
 // on mma.sync (w kept in BF16 as a [W][edge] tile), then the work units.
 #include "conv_common.cuh"
+#include "async_copy.cuh"
 
 namespace sn {
 
@@ -51,41 +52,6 @@ struct TcSets {
     static constexpr PathSets sets = tc_path_sets(L1, LMAX, KIND);
 };
 
-// ---- bulk copies (the TMA engine's linear mode) completed on an mbarrier
-__device__ __forceinline__ void mbar_init(uint64_t* bar, unsigned count) {
-    const unsigned a = (unsigned)__cvta_generic_to_shared(bar);
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(a), "r"(count) : "memory");
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, unsigned bytes) {
-    const unsigned a = (unsigned)__cvta_generic_to_shared(bar);
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(a), "r"(bytes) : "memory");
-}
-
-// global -> shared, `bytes` a multiple of 16 and both addresses 16-byte aligned
-__device__ __forceinline__ void bulk_copy(void* dst, const void* src, unsigned bytes, uint64_t* bar) {
-    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    const unsigned b = (unsigned)__cvta_generic_to_shared(bar);
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
-                 ::"r"(d), "l"(src), "r"(bytes), "r"(b) : "memory");
-}
-
-// Wait for phase `parity` of the barrier to complete, for at most about `limit`
-// clock cycles; false when the limit ran out.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, long long limit) {
-    const unsigned a = (unsigned)__cvta_generic_to_shared(bar);
-    const long long t0 = clock64();
-    while (true) {
-        unsigned done;
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-                     " selp.u32 %0, 1, 0, p;\n}\n" : "=r"(done) : "r"(a), "r"(parity) : "memory");
-        if (done) return true;
-        if (clock64() - t0 > limit) return false;
-    }
-}
-
-constexpr long long TC_WAIT_LIMIT = 4000000000LL;   // about two seconds at 2 GHz
 
 __device__ __forceinline__ uint32_t bf2_bits(__nv_bfloat162 v) { return *reinterpret_cast<uint32_t*>(&v); }
 __device__ __forceinline__ __nv_bfloat162 bits_bf2(uint32_t v) { return *reinterpret_cast<__nv_bfloat162*>(&v); }
@@ -439,11 +405,11 @@ conv_fwd_tc_kernel(const ConvDesc D, const float* __restrict__ W1, const __nv_bf
         tc_w_gemm<H>(D, L, smem, W3T_h);
         // the x rows have landed (bounded wait: a copy that never completes is
         // reported in flags[FLAG_COPY_TIMEOUT] and the CTA's messages are left NaN)
-        const bool ok = mbar_wait(&s_bar, parity, TC_WAIT_LIMIT);
+        const bool ok = mbar_wait(&s_bar, parity, BULK_WAIT_LIMIT);
         parity ^= 1u;
         if (__syncthreads_or(!ok)) {
             if (t == 0 && flags) atomicOr(flags + FLAG_COPY_TIMEOUT, 1);
-            mbar_wait(&s_bar, parity ^ 1u, TC_WAIT_LIMIT);          // once more for the copies in flight
+            mbar_wait(&s_bar, parity ^ 1u, BULK_WAIT_LIMIT);          // once more for the copies in flight
             for (int v = v0 + warp; v < v1; v += CONV_WARPS)
                 for (int i = lane; i < D.m_dim; i += 32) m[(size_t)v * D.m_dim + i] = __int_as_float(0x7fc00000);
             return;

@@ -13,6 +13,7 @@ include/sevennet.h:
 For each coupling (l1, l2, l3) with l <= LMAX it writes a specialisation
     CG<l1,l2,l3>::G(Y, G)        G[m1][m3] = sum_m2 C[m1,m2,m3] Y[m2]
     CG<l1,l2,l3>::gY(a, b, gY)   gY[m2] += sum_{m1,m3} C[m1,m2,m3] a[m1] b[m3]
+    CG<l1,l2,l3>::M(T, m)        m[m3] = sum_{m1,m2} C[m1,m2,m3] T[m1][m2]
 with every structurally zero coefficient dropped.
 """
 
@@ -146,6 +147,12 @@ def emit(path):
                     if terms:
                         expr = " + ".join(f"{_lit(v)} * (a[{a}] * b[{c}])" for a, c, v in terms)
                         lines.append(f"    gy[{bb}] += {expr};")
+                lines.append("  }")
+                lines.append("  static __device__ __forceinline__ void M(const float* __restrict__ T, float* __restrict__ m) {")
+                for c in range(n3):
+                    terms = [(a, b, v) for (a, b, cc), v in sorted(tab.items()) if cc == c]
+                    expr = " + ".join(f"{_lit(v)} * T[{a * (2 * l2 + 1) + b}]" for a, b, v in terms)
+                    lines.append(f"    m[{c}] = {expr};")
                 lines.append("  }")
                 lines.append("};")
                 lines.append("")

@@ -193,6 +193,90 @@ __host__ __device__ constexpr PathSets tc_path_sets(int l1, int lmax, int kind) 
     return s;
 }
 
+// Streaming forward (conv_fwd_stream.cu): a consumer warp owns one set of paths
+// of one input irrep over 32 channels and keeps, per receiver, the sums over
+// edges of w x_{m1} Y_{m2} in registers.  Multiply-adds per channel and edge of a
+// path in that form, and the sums it keeps.  l2 = 0 has one harmonic (1); the
+// scalar product l3 = 0 contracts x with Y first (its coupling is diagonal).
+__host__ __device__ constexpr int st_path_cost(int l1, int l2, int l3) {
+    const int n1 = 2 * l1 + 1, n2 = 2 * l2 + 1;
+    return l2 == 0 ? n1 : (l1 == 0 ? 1 + n2 : (l3 == 0 ? n1 + 1 : n1 * (1 + n2)));
+}
+__host__ __device__ constexpr int st_path_acc(int l1, int l2, int l3) {
+    const int n1 = 2 * l1 + 1, n2 = 2 * l2 + 1;
+    return l2 == 0 ? n1 : (l1 == 0 ? n2 : (l3 == 0 ? 1 : n1 * n2));
+}
+
+// Path sets of one input irrep: largest path first into the set with the least
+// work, at most ST_TILES paths a set, as many sets as keep a set near ST_CAP
+// multiply-adds (the SM's four sub-partitions then carry about the same work).
+constexpr int ST_TILES = 3, ST_CAP = 34, ST_MAX_SETS = 8;
+struct StSets {
+    int n;
+    int cnt[ST_MAX_SETS];
+    int path[ST_MAX_SETS][ST_TILES];     // index into path_list(l1, lmax, kind)
+};
+__host__ __device__ constexpr StSets st_sets(int l1, int lmax, int kind) {
+    StSets s{};
+    const PathList p = path_list(l1, lmax, kind);
+    if (p.n == 0) return s;
+    int total = 0, top = ST_CAP;
+    for (int i = 0; i < p.n; ++i) {
+        const int c = st_path_cost(l1, p.l2[i], p.l3[i]);
+        total += c;
+        top = c > top ? c : top;
+    }
+    int n = (total + top - 1) / top;
+    const int least = (p.n + ST_TILES - 1) / ST_TILES;
+    s.n = n > least ? n : least;
+    int load[ST_MAX_SETS] = {};
+    bool done[12] = {};
+    for (int k = 0; k < p.n; ++k) {
+        int big = -1;
+        for (int i = 0; i < p.n; ++i)
+            if (!done[i] && (big < 0 || st_path_cost(l1, p.l2[i], p.l3[i]) > st_path_cost(l1, p.l2[big], p.l3[big])))
+                big = i;
+        done[big] = true;
+        int at = -1;
+        for (int j = 0; j < s.n; ++j)
+            if (s.cnt[j] < ST_TILES && (at < 0 || load[j] < load[at])) at = j;
+        s.path[at][s.cnt[at]++] = big;
+        load[at] += st_path_cost(l1, p.l2[big], p.l3[big]);
+    }
+    return s;
+}
+__host__ __device__ constexpr int st_set_cost(int l1, int lmax, int kind, int j) {
+    const PathList p = path_list(l1, lmax, kind);
+    const StSets s = st_sets(l1, lmax, kind);
+    int c = 0;
+    for (int i = 0; i < s.cnt[j]; ++i) c += st_path_cost(l1, p.l2[s.path[j][i]], p.l3[s.path[j][i]]);
+    return c;
+}
+
+// One CTA type of the streaming forward: up to four units (one per quarter of the
+// 128 TMEM lanes), the W3 rows they need as the MMA's A operand, and the pieces
+// of an x row they read.
+struct StUnit {
+    int16_t l1, set, group, n_paths;
+    int32_t xoff, xstep;                 // floats: first channel in a staged x row, step between components
+    int16_t n3[4];                       // 2 l3 + 1 of each path
+    int32_t m_off[ST_TILES], m_mul[ST_TILES];   // message row: first channel of each path, step between components
+};
+struct StType {
+    int16_t n_units, tiles, n_seg, pad;
+    int32_t row_floats;                  // floats of a staged x row
+    int32_t seg_src[4], seg_dst[4], seg_n[4], seg_step[4], seg_floats[4];   // pieces: n copies of seg_floats, step in x
+    int32_t cta0, n_cta;
+    const void* w3;                      // [3 terms][tiles][128 rows][64] BF16
+    StUnit u[4];
+};
+constexpr int ST_MAX_TYPES = 16;
+struct StPlan {
+    int32_t n_types, n_cta, stages, ok;
+    int32_t smem;                        // bytes of dynamic shared memory
+    StType t[ST_MAX_TYPES];
+};
+
 struct PathDesc {
     int32_t l1, l2, l3, kind;
     int32_t mul;      // channels of the path (= multiplicity of l1 in the block input)
@@ -260,6 +344,7 @@ struct GemmBatch {
 
 struct LayerDev {
     ConvDesc conv;
+    StPlan st[2];                 // streaming forward, FP32 and BF16
     int x_dim, y_dim, h_in_dim, h_out_dim, m_dim;
     int in_mul[NL], y_mul[NL], msg_mul[NL], out_mul[NL];
     int in_off[NL], y_off[NL], msg_off[NL], out_off[NL];
@@ -271,6 +356,7 @@ struct LayerDev {
     float* mlp0T = nullptr;  // [H][NB]
     float* mlp1T = nullptr;  // [H][H]
     float* mlp2T = nullptr;  // [W][H]
+    uint2* mlp1F = nullptr;  // W2 as B fragments, three BF16 terms (radial.cu)
     __nv_bfloat16* mlp1h = nullptr;   // [2][H][H] W2 as stored, hi then lo (B operand of gA2 @ W2^T)
     __nv_bfloat16* mlp1Th = nullptr;  // [2][H][H] W2^T, hi then lo (B operand of H1 @ W2)
     __nv_bfloat16* mlp2h = nullptr;   // [W][H]  (N-major for mma B operand)
@@ -305,6 +391,7 @@ struct sevennet_model {
     std::vector<double> shift;
     int T = 0, lmax = 0, H = 0, NB = 0;
     int h_max = 0, x_max = 0, y_max = 0, m_max = 0;
+    int h2_bytes = 0;           // hidden activations per pair for the streaming forward (0: not used)
     std::vector<sn::LayerDev> layers;
     float* embed = nullptr;     // [n_species][mul0]
     float* readout = nullptr;   // [mul0] = scale * R0 R1 / sqrt(mul0 hid)
@@ -340,6 +427,9 @@ struct Workspace {
     float4* geom = nullptr;       // [E] (d, r)
     // unordered pairs {e, rev[e]} with e < rev[e], in receiver order (the adjoint's units)
     int* pair_ptr = nullptr;      // [N+1] pairs of receivers < v; pair_ptr[N] = number of pairs
+    int* quad_ptr = nullptr;      // [N+1] groups of four edges of receivers < v
+    int2* quads = nullptr;        // [E/4 + N] (first edge, receiver | (edges - 1) << 29)
+    int64_t cap_quads = 0;
     int* p_e = nullptr;           // [E] edge of each pair
     int* p_dst = nullptr;         // [E] its receiver
     int* p_src = nullptr;         // [E] its sender
@@ -350,6 +440,10 @@ struct Workspace {
     int* sdesc = nullptr;         // [S][16] bins, offsets, search ranges, pbc
     int64_t* atom_off = nullptr;  // [S+1]
     // model activations
+    // One block of memory holds gxq, gx, gy, gh and h, in this order; the forward keeps
+    // the pairs' hidden activations there while a convolution runs (all five are dead then)
+    unsigned char* grad = nullptr;
+    int64_t grad_bytes = 0;
     float* h = nullptr;           // [N][h_max]
     float* xs = nullptr;          // [T][N][x_max]
     float* ys = nullptr;          // [T][N][y_max]
@@ -407,7 +501,7 @@ sevennet_status refresh_neighbors(sevennet_model* M, Workspace* ws, int64_t n_at
 // the workspace's graph.
 void model_embed(sevennet_model* M, Workspace* ws, int64_t N, cudaStream_t st);
 void model_layer_forward(sevennet_model* M, Workspace* ws, int t, int64_t N, int64_t E,
-                         sevennet_precision prec, cudaStream_t st);
+                         sevennet_precision prec, cudaStream_t st, bool pairs = false);
 void model_readout(sevennet_model* M, Workspace* ws, int64_t N, cudaStream_t st);
 void model_layer_backward_gate(sevennet_model* M, Workspace* ws, int t, int64_t N, cudaStream_t st);
 // pairs: the convolution adjoint runs over ws's pair list (built by build_pairs
@@ -460,6 +554,23 @@ sevennet_status conv_configure_fwd_tc(int H, size_t need);
 void launch_conv_fwd_tc(const LayerDev& L, int H, int64_t n_atoms, int64_t n_edges, const int* row_ptr,
                         const int* dst, const int* src, const float4* geom, const float* x, float* m,
                         int* flags, cudaStream_t st);
+// Streaming forward over a symmetric list with its pairs (conv_fwd_stream.cu).
+// h2: hidden activations of the radial MLP per pair (launch_radial), 64 values a
+// pair: FP32, or BF16 in the BF16 path; pair_of: the pair of every edge.
+sevennet_status st_plan_build(sevennet_model* M, LayerDev& L);
+sevennet_status radial_pack(sevennet_model* M, LayerDev& L);
+int st_h2_bytes(const sevennet_model* M);
+int64_t st_grad_bytes(const sevennet_model* M);     // gradients (and h) of one atom
+sevennet_status st_configure(int lmax);
+void launch_conv_fwd_stream(const LayerDev& L, sevennet_precision prec, int64_t n_atoms, int64_t cap_pairs,
+                            const int* row_ptr, const int* quad_ptr, const int2* quads, const int* src,
+                            const float4* geom, const int* pair_of, const void* h2, const float* x, float* m,
+                            int* flags, cudaStream_t st);
+void launch_quads(int64_t n_atoms, const int* row_ptr, const int* quad_ptr, int2* quads, cudaStream_t st);
+void launch_radial(const LayerDev& L, sevennet_precision prec, int64_t cap_pairs, const int* n_pairs,
+                   const float4* p_geom, void* h2, cudaStream_t st);
+void launch_pair_of(int64_t cap_pairs, int64_t n_atoms, const int* row_ptr, const int* rev, const int* pair_ptr,
+                    const int* p_e, int* pair_of, cudaStream_t st);
 void launch_gemm(const GemmBatch& b, sevennet_precision prec, cudaStream_t st);
 // The adjoint over unordered pairs (ws->pair_ptr / p_*): n_pairs is an upper
 // bound on the pair count (the count is pair_ptr[n_atoms], on the device); the

@@ -59,20 +59,25 @@ __global__ void bin_atoms_kernel(int64_t n, int S, const int64_t* __restrict__ a
     atomicAdd(bin_count + bin, 1);
 }
 
-// Exclusive scan of n ints into out[0..n] (out[n] = total) with one CTA.
-__global__ void __launch_bounds__(1024) scan_kernel(const int* __restrict__ in, int64_t n,
-                                                    int* __restrict__ out, int* __restrict__ total,
-                                                    const int* cond) {
-    if (skip(cond)) return;
+// Exclusive scan of n values f(i) into out[0..n] (out[n] = total) with one CTA:
+// eight consecutive values a thread, 8,192 a round.
+template <typename F>
+__device__ __forceinline__ void cta_scan(int64_t n, F f, int* __restrict__ out, int* __restrict__ total) {
+    constexpr int PER = 8;
     __shared__ int warp_sums[32];
     __shared__ int carry;
     const int t = threadIdx.x, lane = t & 31, w = t >> 5;
-    if (t == 0) carry = 0;
     __syncthreads();
-    for (int64_t base = 0; base < n; base += 1024) {
-        const int64_t i = base + t;
-        const int x = (i < n) ? in[i] : 0;
-        int s = x;
+    if (t == 0) carry = 0;
+    for (int64_t base = 0; base < n; base += 1024 * PER) {
+        const int64_t i0 = base + (int64_t)t * PER;
+        int x[PER], sum = 0;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            x[k] = i0 + k < n ? f(i0 + k) : 0;
+            sum += x[k];
+        }
+        int s = sum;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const int y = __shfl_up_sync(0xffffffffu, s, o);
@@ -90,16 +95,37 @@ __global__ void __launch_bounds__(1024) scan_kernel(const int* __restrict__ in, 
             warp_sums[lane] = ws;
         }
         __syncthreads();
-        const int excl = carry + (w ? warp_sums[w - 1] : 0) + s - x;
-        if (i < n) out[i] = excl;
+        int excl = carry + (w ? warp_sums[w - 1] : 0) + s - sum;
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            if (i0 + k < n) out[i0 + k] = excl;
+            excl += x[k];
+        }
         __syncthreads();
-        if (t == 1023) carry = excl + x;
+        if (t == 1023) carry = excl;
         __syncthreads();
     }
+    __syncthreads();
     if (t == 0) {
         out[n] = carry;
         if (total) *total = carry;
     }
+}
+
+__global__ void __launch_bounds__(1024) scan_kernel(const int* __restrict__ in, int64_t n,
+                                                    int* __restrict__ out, int* __restrict__ total,
+                                                    const int* cond) {
+    if (skip(cond)) return;
+    cta_scan(n, [=](int64_t i) { return in[i]; }, out, total);
+}
+
+// The pair offsets and, in a second CTA, the offsets of the receivers' groups of four edges.
+__global__ void __launch_bounds__(1024) scan_pairs_kernel(const int* __restrict__ cnt, int64_t n,
+                                                          int* __restrict__ pair_ptr,
+                                                          const int* __restrict__ row_ptr,
+                                                          int* __restrict__ quad_ptr) {
+    if (blockIdx.x == 0) cta_scan(n, [=](int64_t i) { return cnt[i]; }, pair_ptr, nullptr);
+    else cta_scan(n, [=](int64_t i) { return (row_ptr[i + 1] - row_ptr[i] + 3) >> 2; }, quad_ptr, nullptr);
 }
 
 __global__ void place_kernel(int64_t n, const int* __restrict__ bin_of, const int* __restrict__ bin_start,
@@ -358,7 +384,7 @@ void build_pairs(Workspace* ws, int64_t N, cudaStream_t st) {
     if (N > 0)
         pairs_kernel<false><<<blocks, 256, 0, st>>>(N, ws->row_ptr, ws->rev, nullptr, nullptr, nullptr, ws->row_cnt,
                                                    nullptr, nullptr, nullptr, nullptr, nullptr);
-    scan_kernel<<<1, 1024, 0, st>>>(ws->row_cnt, N, ws->pair_ptr, nullptr, nullptr);
+    scan_pairs_kernel<<<2, 1024, 0, st>>>(ws->row_cnt, N, ws->pair_ptr, ws->row_ptr, ws->quad_ptr);
     if (N > 0)
         pairs_kernel<true><<<blocks, 256, 0, st>>>(N, ws->row_ptr, ws->rev, ws->dst, ws->src, ws->geom, nullptr,
                                                   ws->pair_ptr, ws->p_e, ws->p_dst, ws->p_src, ws->p_geom);

@@ -494,6 +494,7 @@ sevennet_status ws_reserve(sevennet_model* M, Workspace* ws, int64_t n_atoms, in
         SN_TRY(ws_alloc(ws, &ws->pos_s, N * 3));
         SN_TRY(ws_alloc(ws, &ws->frac_floor, N * 3));
         SN_TRY(ws_alloc(ws, &ws->q32, N));
+        SN_TRY(ws_alloc(ws, &ws->bin_s, N));
         SN_TRY(ws_alloc(ws, &ws->species_s, N));
         SN_TRY(ws_alloc(ws, &ws->row_ptr, N + 1));
         SN_TRY(ws_alloc(ws, &ws->row_cnt, N + 1));
@@ -555,6 +556,12 @@ sevennet_status ws_reserve(sevennet_model* M, Workspace* ws, int64_t n_atoms, in
         SN_TRY(ws_alloc(ws, &ws->sdesc, S * 16));
         SN_TRY(ws_alloc(ws, &ws->atom_off, S + 1));
         ws->cap_structs = S;
+    }
+    const int64_t partials = ws->cap_atoms / 512 + ws->cap_structs + 1;
+    if (partials > ws->cap_partial) {
+        ws->cap_partial = 0;
+        SN_TRY(ws_alloc(ws, &ws->partial, partials * 10));
+        ws->cap_partial = partials;
     }
     return SEVENNET_OK;
 }
@@ -724,10 +731,13 @@ sevennet_status run_model(sevennet_model* M, Workspace* ws, const BatchHost& b, 
     }
     prof_begin(&M->prof, PF_OTHER, st, &ev);
     launch_forces(N, ws->row_ptr, ws->rev, ws->gd, ws->geom, ws->f_s, ws->w_atom, st);
-    launch_reduce_structs(b.n_structs, ws->atom_off, ws->e_atom, ws->w_atom, energy_dev, virial_dev, st);
+    int64_t max_atoms = 0;
+    for (int s = 0; s < b.n_structs; ++s) max_atoms = std::max(max_atoms, b.atom_off[s + 1] - b.atom_off[s]);
+    launch_reduce_structs(b.n_structs, max_atoms, ws->atom_off, ws->e_atom, ws->w_atom, ws->partial, energy_dev,
+                          virial_dev, st);
     launch_scatter_forces(N, ws->perm, ws->f_s, forces_dev, st);
-    prof_end(&M->prof, PF_OTHER, st, ev, 3);
-    count_launches(3);
+    prof_end(&M->prof, PF_OTHER, st, ev, 4);
+    count_launches(4);
     SN_CUDA(cudaGetLastError());
     return SEVENNET_OK;
 }

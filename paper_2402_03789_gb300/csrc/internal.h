@@ -415,7 +415,9 @@ struct Workspace {
     int* perm = nullptr;          // [N] internal -> input index
     int* struct_of = nullptr;     // [N] internal atom -> structure
     double* pos_s = nullptr;      // [N][3] wrapped positions in internal order
-    double* frac_floor = nullptr; // [N][3] integer image of each internal atom
+    int* frac_floor = nullptr;    // [N][3] integer image of each internal atom
+    int* bin_s = nullptr;         // [N] bin of each internal atom
+    double* partial = nullptr;    // [N / 512 + S + 1][10] partial energy and virial sums
     float4* q32 = nullptr;        // [N] wrapped positions in FP32 (distance pre-test)
     int* species_s = nullptr;     // [N]
     int* row_ptr = nullptr;       // [N+1]
@@ -429,7 +431,7 @@ struct Workspace {
     int* pair_ptr = nullptr;      // [N+1] pairs of receivers < v; pair_ptr[N] = number of pairs
     int* quad_ptr = nullptr;      // [N+1] groups of four edges of receivers < v
     int2* quads = nullptr;        // [E/4 + N] (first edge, receiver | (edges - 1) << 29)
-    int64_t cap_quads = 0;
+    int64_t cap_quads = 0, cap_partial = 0;
     int* p_e = nullptr;           // [E] edge of each pair
     int* p_dst = nullptr;         // [E] its receiver
     int* p_src = nullptr;         // [E] its sender
@@ -593,8 +595,8 @@ void launch_readout(const float* h, int h_dim, const float* c, const double* shi
                     const int* species, int64_t n, int mul0, int n_species, double* e_atom, cudaStream_t st);
 void launch_forces(int64_t n, const int* row_ptr, const int* rev, const float* gd,
                    const float4* geom, double* f_s, double* w_atom, cudaStream_t st);
-void launch_reduce_structs(int32_t n_structs, const int64_t* atom_off, const double* e_atom,
-                           const double* w_atom, double* energy, double* virial, cudaStream_t st);
+void launch_reduce_structs(int32_t n_structs, int64_t max_atoms, const int64_t* atom_off, const double* e_atom,
+                           const double* w_atom, double* partial, double* energy, double* virial, cudaStream_t st);
 void launch_scatter_forces(int64_t n, const int* perm, const double* f_s, double* forces,
                            cudaStream_t st);
 

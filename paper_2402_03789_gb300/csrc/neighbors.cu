@@ -161,8 +161,9 @@ __global__ void gather_kernel(int64_t n, int S, const int64_t* __restrict__ atom
                               const int* __restrict__ sdesc, const double* __restrict__ cells,
                               const double* __restrict__ inv_cells, const int* __restrict__ perm,
                               const double* __restrict__ pos, const int32_t* __restrict__ species,
-                              double* __restrict__ pos_s, double* __restrict__ fl_s, float4* __restrict__ q32,
-                              int* __restrict__ species_s, int* __restrict__ struct_of, const int* cond) {
+                              double* __restrict__ pos_s, int* __restrict__ fl_s, float4* __restrict__ q32,
+                              int* __restrict__ species_s, int* __restrict__ struct_of,
+                              const int* __restrict__ bin_of, int* __restrict__ bin_s, const int* cond) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n || skip(cond)) return;
     const int64_t o = perm[i];
@@ -175,7 +176,7 @@ __global__ void gather_kernel(int64_t n, int S, const int64_t* __restrict__ atom
     for (int a = 0; a < 3; ++a) {
         double f = p[0] * ic[0 * 3 + a] + p[1] * ic[1 * 3 + a] + p[2] * ic[2 * 3 + a];
         fl[a] = d[6 + a] ? floor(f) : 0.0;
-        fl_s[i * 3 + a] = fl[a];
+        fl_s[i * 3 + a] = (int)fl[a];
     }
     const double* c = cells + s * 9;
     double q[3];
@@ -187,35 +188,39 @@ __global__ void gather_kernel(int64_t n, int S, const int64_t* __restrict__ atom
     q32[i] = make_float4((float)q[0], (float)q[1], (float)q[2], 0.0f);
     species_s[i] = species[o];
     struct_of[i] = s;
+    bin_s[i] = bin_of[o];
 }
 
 // Count (FILL = false) or write (FILL = true) the edges of every internal atom
-// v.  A group of NGL lanes serves one receiver: it scans the bins within the
-// search range in a fixed order, the members of a bin in order, NGL candidates
-// at a time; a ballot over the group gives each hit its slot, so the edge order
-// is the serial one (bin order, then member order).  d = q_w - q_v + S~ cell,
-// with q the wrapped positions; the edge's shift is S~ - n_w + n_v.  The test
-// that decides an edge is FP64.  An FP32 pre-test skips the FP64 work for
+// v, a warp per receiver.  The lanes look up the bins within the search range, 32
+// at a time; the members of those bins then form one list in bin order, member
+// order, of which every lane tests one candidate, so the edge order is the serial
+// one.  d = q_w - q_v + S~ cell, with q the wrapped positions; the edge's shift is
+// S~ - n_w + n_v.  The test that decides an edge is FP64.  An FP32 pre-test drops
 // candidates clearly outside r_c; its margin, 1e-3 A + 1e-6 (|q_v| + |S~ cell| +
 // r_c), is over ten times the FP32 rounding of d for any coordinates (positions
-// along non-periodic directions are not wrapped), so it cannot drop an edge.
-constexpr int NGL = 2;
+// along non-periodic directions are not wrapped), so it cannot drop an edge.  What
+// passes is queued in shared memory, so that the FP64 instructions (a few lanes of
+// FP64 a sub-partition) run on full warps: 24,000 atoms, both passes, 595 us with
+// two lanes walking a receiver's bins one after another.
+constexpr int EDGE_WARPS = 4;
+constexpr int NGL = 2;              // lanes per receiver of the list refresh
 
 __device__ __forceinline__ int floor_div(int a, int n) { return a >= 0 ? a / n : -((n - 1 - a) / n); }
 
 template <bool FILL>
-__global__ void __launch_bounds__(128)
+__global__ void __launch_bounds__(EDGE_WARPS * 32)
 edges_kernel(int64_t n, double rc2, float rc32, int64_t cap, const int* __restrict__ sdesc,
              const double* __restrict__ cells, const int* __restrict__ struct_of, const int* __restrict__ bin_start,
-             const double* __restrict__ q_s, const float4* __restrict__ q32, const double* __restrict__ fl_s,
-             const int* __restrict__ row_ptr,
+             const int* __restrict__ bin_s, const double* __restrict__ q_s, const float4* __restrict__ q32,
+             const int* __restrict__ fl_s, const int* __restrict__ row_ptr,
              int* __restrict__ counts, int* __restrict__ flags, int* __restrict__ dst, int* __restrict__ src,
              int* __restrict__ shift, float4* __restrict__ geom, const int* cond) {
-    const int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / NGL;
-    if (v >= n || skip(cond)) return;                      // the whole group leaves together
-    const int j = threadIdx.x & (NGL - 1);
-    const int gsh = threadIdx.x & 31 & ~(NGL - 1);
-    const unsigned gmask = ((1u << NGL) - 1) << gsh;
+    __shared__ int2 s_queue[EDGE_WARPS][64];              // (sender, packed image) of candidates that passed
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t v = (int64_t)blockIdx.x * EDGE_WARPS + warp;
+    if (v >= n || skip(cond)) return;                      // whole warps
+    int2* queue = s_queue[warp];
     const int s = struct_of[v];
     const int* d = sdesc + s * SD;
     const double* c = cells + s * 9;
@@ -225,86 +230,120 @@ edges_kernel(int64_t n, double rc2, float rc32, int64_t cap, const int* __restri
     float c32[9];
 #pragma unroll
     for (int a = 0; a < 9; ++a) c32[a] = (float)c[a];
-    int bv[3];
-    {
-        const int base = d[9];
-        const int nb = d[0] * d[1] * d[2];
-        int lo = base, hi = base + nb;   // largest b with bin_start[b] <= v
-        while (hi - lo > 1) {
-            const int mid = (lo + hi) >> 1;
-            if (bin_start[mid] <= v) lo = mid; else hi = mid;
-        }
-        const int local = lo - base;
-        bv[2] = local % d[2];
-        bv[1] = (local / d[2]) % d[1];
-        bv[0] = local / (d[2] * d[1]);
-    }
+    const int d0 = d[0], d1 = d[1], d2 = d[2], base = d[9];
+    const int k0 = d[3], k1 = d[4], k2 = d[5], w1 = 2 * k1 + 1, w2 = 2 * k2 + 1;
+    const int n_near = (2 * k0 + 1) * w1 * w2;             // bins in range
+    const int local = bin_s[v] - base;
+    const int bv[3] = {local / (d2 * d1), (local / d2) % d1, local % d2};
     int64_t e = FILL ? (int64_t)row_ptr[v] : 0;
+    int flv[3] = {0, 0, 0};
+    if constexpr (FILL) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) flv[a] = fl_s[v * 3 + a];
+    }
     bool close = false;
-    for (int ox = -d[3]; ox <= d[3]; ++ox) {
-        int bx = bv[0] + ox, sx = 0;
-        if (d[6]) { sx = floor_div(bx, d[0]); bx -= sx * d[0]; }
-        else if (bx < 0 || bx >= d[0]) continue;
-        for (int oy = -d[4]; oy <= d[4]; ++oy) {
-            int by = bv[1] + oy, sy = 0;
-            if (d[7]) { sy = floor_div(by, d[1]); by -= sy * d[1]; }
-            else if (by < 0 || by >= d[1]) continue;
-            for (int oz = -d[5]; oz <= d[5]; ++oz) {
-                int bz = bv[2] + oz, sz = 0;
-                if (d[8]) { sz = floor_div(bz, d[2]); bz -= sz * d[2]; }
-                else if (bz < 0 || bz >= d[2]) continue;
-                const int b = d[9] + (bx * d[1] + by) * d[2] + bz;
-                const float fx = (float)sx, fy = (float)sy, fz = (float)sz;
+    int qn = 0;
+    // FP64 test of the first m (<= 32) queued candidates, in order
+    auto drain = [&](int m) {
+        __syncwarp();
+        const bool in = lane < m;
+        const int2 cand = queue[in ? lane : 0];
+        const int w = cand.x;
+        const int sx = (cand.y & 1023) - 512, sy = ((cand.y >> 10) & 1023) - 512, sz = ((cand.y >> 20) & 1023) - 512;
+        double dd[3], r2 = 0.0;
+#pragma unroll
+        for (int a = 0; a < 3; ++a) dd[a] = q_s[(int64_t)w * 3 + a] - qv[a];
+        if (__any_sync(0xffffffffu, (sx | sy | sz) != 0)) {
+#pragma unroll
+            for (int a = 0; a < 3; ++a) dd[a] += sx * c[a] + sy * c[3 + a] + sz * c[6 + a];
+        }
+        r2 = dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2];
+        const bool self = w == v && sx == 0 && sy == 0 && sz == 0;
+        const bool hit = in && !self && r2 < rc2;
+        const unsigned mine = __ballot_sync(0xffffffffu, hit);
+        if constexpr (FILL) {
+            const int64_t slot = e + __popc(mine & ((1u << lane) - 1u));
+            if (hit && slot < cap) {
+                dst[slot] = (int)v;
+                src[slot] = w;
+                shift[slot * 3 + 0] = sx - fl_s[w * 3 + 0] + flv[0];
+                shift[slot * 3 + 1] = sy - fl_s[w * 3 + 1] + flv[1];
+                shift[slot * 3 + 2] = sz - fl_s[w * 3 + 2] + flv[2];
+                // |d|: an FP32 root corrected by its FP64 remainder (right to the last bit but
+                // for near ties; the FP64 root took most of the pass)
+                const float rt = sqrtf((float)r2);
+                geom[slot] = make_float4((float)dd[0], (float)dd[1], (float)dd[2],
+                                         fmaf((float)fma(-(double)rt, (double)rt, r2), 0.5f / rt, rt));
+            }
+        } else {
+            if (hit && r2 < 1e-16) close = true;
+        }
+        e += __popc(mine);
+        const int2 rest = queue[lane + 32 < 64 ? lane + 32 : 63];
+        __syncwarp();
+        qn -= m;
+        if (lane < qn) queue[lane] = rest;
+        __syncwarp();
+    };
+    for (int b0 = 0; b0 < n_near; b0 += 32) {
+        const int i = b0 + lane;
+        int start = 0, cnt = 0, img = 0;
+        if (i < n_near) {
+            int bx = bv[0] + i / (w1 * w2) - k0, by = bv[1] + (i / w2) % w1 - k1, bz = bv[2] + i % w2 - k2;
+            int sx = 0, sy = 0, sz = 0;
+            bool ok = true;
+            if (d[6]) { sx = floor_div(bx, d0); bx -= sx * d0; } else ok = ok && bx >= 0 && bx < d0;
+            if (d[7]) { sy = floor_div(by, d1); by -= sy * d1; } else ok = ok && by >= 0 && by < d1;
+            if (d[8]) { sz = floor_div(bz, d2); bz -= sz * d2; } else ok = ok && bz >= 0 && bz < d2;
+            if (ok) {
+                const int b = base + (bx * d1 + by) * d2 + bz;
+                start = bin_start[b];
+                cnt = bin_start[b + 1] - start;
+                img = (sx + 512) | ((sy + 512) << 10) | ((sz + 512) << 20);
+            }
+        }
+        int incl = cnt;                                    // members of the bins up to this lane's
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += y;
+        }
+        const int total = __shfl_sync(0xffffffffu, incl, 31);
+        for (int t0 = 0; t0 < total; t0 += 32) {
+            const int t = t0 + lane;
+            int j = 0;                                     // first bin whose members reach past t
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                const int y = __shfl_sync(0xffffffffu, incl, j + o - 1);
+                if (y <= t) j += o;
+            }
+            j = min(j, 31);
+            const int before = __shfl_sync(0xffffffffu, incl - cnt, j), st = __shfl_sync(0xffffffffu, start, j);
+            const int im = __shfl_sync(0xffffffffu, img, j);
+            bool pass = false;
+            int w = 0;
+            if (t < total) {
+                w = st + t - before;
+                const float fx = (float)((im & 1023) - 512), fy = (float)(((im >> 10) & 1023) - 512),
+                            fz = (float)(((im >> 20) & 1023) - 512);
                 const float sh32[3] = {fx * c32[0] + fy * c32[3] + fz * c32[6],
                                        fx * c32[1] + fy * c32[4] + fz * c32[7],
                                        fx * c32[2] + fy * c32[5] + fz * c32[8]};
                 const float smag = fmaxf(fabsf(sh32[0]), fmaxf(fabsf(sh32[1]), fabsf(sh32[2])));
                 const float rpre = rc32 + 1e-3f + 1e-6f * (qmag + smag + rc32);
-                const float rc2_pre = rpre * rpre;
-                const int w1 = bin_start[b + 1];
-                for (int w0 = bin_start[b]; w0 < w1; w0 += NGL) {
-                    const int w = w0 + j;
-                    bool hit = false;
-                    double dd[3], r2 = 0.0;
-                    if (w < w1) {
-                        const float4 qw = q32[w];
-                        const float ex = qw.x - qv32.x + sh32[0], ey = qw.y - qv32.y + sh32[1],
-                                    ez = qw.z - qv32.z + sh32[2];
-                        if (ex * ex + ey * ey + ez * ez < rc2_pre) {
-                            const double sh[3] = {
-                                sx * c[0] + sy * c[3] + sz * c[6],
-                                sx * c[1] + sy * c[4] + sz * c[7],
-                                sx * c[2] + sy * c[5] + sz * c[8]};
-#pragma unroll
-                            for (int a = 0; a < 3; ++a) dd[a] = q_s[w * 3 + a] - qv[a] + sh[a];
-                            r2 = dd[0] * dd[0] + dd[1] * dd[1] + dd[2] * dd[2];
-                            const bool self = (w == v) && sx == 0 && sy == 0 && sz == 0;
-                            hit = !self && r2 < rc2;
-                        }
-                    }
-                    const unsigned mine = (__ballot_sync(gmask, hit) >> gsh) & ((1u << NGL) - 1);
-                    if constexpr (FILL) {
-                        if (hit) {
-                            const int64_t slot = e + __popc(mine & ((1u << j) - 1));
-                            if (slot < cap) {
-                                dst[slot] = (int)v;
-                                src[slot] = w;
-                                shift[slot * 3 + 0] = sx - (int)fl_s[w * 3 + 0] + (int)fl_s[v * 3 + 0];
-                                shift[slot * 3 + 1] = sy - (int)fl_s[w * 3 + 1] + (int)fl_s[v * 3 + 1];
-                                shift[slot * 3 + 2] = sz - (int)fl_s[w * 3 + 2] + (int)fl_s[v * 3 + 2];
-                                geom[slot] = make_float4((float)dd[0], (float)dd[1], (float)dd[2], (float)sqrt(r2));
-                            }
-                        }
-                    } else {
-                        if (hit && r2 < 1e-16) close = true;
-                    }
-                    e += __popc(mine);
-                }
+                const float4 qw = q32[w];
+                const float ex = qw.x - qv32.x + sh32[0], ey = qw.y - qv32.y + sh32[1], ez = qw.z - qv32.z + sh32[2];
+                pass = ex * ex + ey * ey + ez * ez < rpre * rpre;
             }
+            const unsigned m = __ballot_sync(0xffffffffu, pass);
+            if (pass) queue[qn + __popc(m & ((1u << lane) - 1u))] = make_int2(w, im);
+            qn += __popc(m);
+            if (qn >= 32) drain(32);
         }
     }
+    if (qn > 0) drain(qn);
     if constexpr (!FILL) {
-        if (j == 0) counts[v] = (int)e;
+        if (lane == 0) counts[v] = (int)e;
         if (close) atomicOr(flags + 1, 1);
     }
 }
@@ -478,9 +517,9 @@ sevennet_status build_neighbors(sevennet_model* M, Workspace* ws, const BatchHos
         gather_kernel<<<blocks_for(N, 256), 256, 0, st>>>(N, S, ws->atom_off, ws->sdesc, ws->cells,
                                                          ws->inv_cells, ws->perm, pos_dev, species_dev,
                                                          ws->pos_s, ws->frac_floor, ws->q32, ws->species_s,
-                                                         ws->struct_of, cond);
-        edges_kernel<false><<<blocks_for(N * NGL, 128), 128, 0, st>>>(
-            N, rc * rc, (float)rc, 0, ws->sdesc, ws->cells, ws->struct_of, ws->bin_start, ws->pos_s, ws->q32,
+                                                         ws->struct_of, ws->bin_of, ws->bin_s, cond);
+        edges_kernel<false><<<blocks_for(N, EDGE_WARPS), EDGE_WARPS * 32, 0, st>>>(
+            N, rc * rc, (float)rc, 0, ws->sdesc, ws->cells, ws->struct_of, ws->bin_start, ws->bin_s, ws->pos_s, ws->q32,
             ws->frac_floor, nullptr, ws->row_cnt, ws->flags, nullptr, nullptr, nullptr, nullptr, cond);
     }
     scan_kernel<<<1, 1024, 0, st>>>(ws->row_cnt, N, ws->row_ptr, ws->flags + 0, cond);
@@ -493,8 +532,8 @@ sevennet_status build_neighbors(sevennet_model* M, Workspace* ws, const BatchHos
         if (E > ws->cap_edges) SN_TRY(ws_reserve(M, ws, N, E + E / 4 + 1024, n_bins, S, st));
     }
     if (N > 0) {
-        edges_kernel<true><<<blocks_for(N * NGL, 128), 128, 0, st>>>(
-            N, rc * rc, (float)rc, ws->cap_edges, ws->sdesc, ws->cells, ws->struct_of, ws->bin_start, ws->pos_s,
+        edges_kernel<true><<<blocks_for(N, EDGE_WARPS), EDGE_WARPS * 32, 0, st>>>(
+            N, rc * rc, (float)rc, ws->cap_edges, ws->sdesc, ws->cells, ws->struct_of, ws->bin_start, ws->bin_s, ws->pos_s,
             ws->q32, ws->frac_floor, ws->row_ptr, nullptr, ws->flags, ws->dst, ws->src, ws->shift, ws->geom, cond);
         clamp_rows_kernel<<<blocks_for(N + 1, 256), 256, 0, st>>>(N, ws->row_ptr, ws->cap_edges, ws->flags, cond);
     }

@@ -10,6 +10,8 @@
 //    -sum_e F_e (x) d_e, both summed in FP64.
 #include "internal.h"
 
+#include <algorithm>
+
 namespace sn {
 
 __device__ __forceinline__ float sigm(float x) { return 1.0f / (1.0f + expf(-x)); }
@@ -383,45 +385,53 @@ void launch_readout(const float* h, int h_dim, const float* c, const double* shi
 }
 
 // ---------------------------------------------------------------- forces / virial
-__global__ void forces_kernel(int64_t n, const int* __restrict__ row_ptr, const int* __restrict__ rev,
-                              const float* __restrict__ gd, const float4* __restrict__ geom,
-                              double* __restrict__ f, double* __restrict__ w) {
-    const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (v >= n) return;
-    double fx = 0, fy = 0, fz = 0;
-    double wv[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-    for (int e = row_ptr[v]; e < row_ptr[v + 1]; ++e) {
-        const float* g = gd + (int64_t)e * 3;
-        const float* gr = gd + (int64_t)rev[e] * 3;
-        const double g0 = g[0], g1 = g[1], g2 = g[2];
-        fx += g0 - (double)gr[0];
-        fy += g1 - (double)gr[1];
-        fz += g2 - (double)gr[2];
-        const float4 d = geom[e];
-        const double dd[3] = {d.x, d.y, d.z};
-        const double gg[3] = {g0, g1, g2};
+// Eight lanes an atom (one walked its edges one after another: 41 us for any cell
+// up to some thousand atoms); each sums every eighth edge, then a fixed tree.
+constexpr int FL = 8;
+
+__global__ void __launch_bounds__(128)
+forces_kernel(int64_t n, const int* __restrict__ row_ptr, const int* __restrict__ rev,
+              const float* __restrict__ gd, const float4* __restrict__ geom,
+              double* __restrict__ f, double* __restrict__ w) {
+    const int64_t v = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / FL;
+    const int j = threadIdx.x & (FL - 1);
+    double acc[12] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0, 0};      // force, then virial
+    if (v < n)
+        for (int e = row_ptr[v] + j; e < row_ptr[v + 1]; e += FL) {
+            const float* g = gd + (int64_t)e * 3;
+            const float* gr = gd + (int64_t)rev[e] * 3;
+            const float4 d = geom[e];
+            const double gg[3] = {g[0], g[1], g[2]}, dd[3] = {d.x, d.y, d.z};
 #pragma unroll
-        for (int a = 0; a < 3; ++a)
+            for (int a = 0; a < 3; ++a) {
+                acc[a] += gg[a] - (double)gr[a];
 #pragma unroll
-            for (int b = 0; b < 3; ++b) wv[a * 3 + b] -= gg[a] * dd[b];
+                for (int b = 0; b < 3; ++b) acc[3 + a * 3 + b] -= gg[a] * dd[b];
+            }
+        }
+#pragma unroll
+    for (int k = 0; k < 12; ++k)
+#pragma unroll
+        for (int o = FL / 2; o > 0; o >>= 1) acc[k] += __shfl_xor_sync(0xffffffffu, acc[k], o);
+    if (v < n && j == 0) {
+#pragma unroll
+        for (int k = 0; k < 3; ++k) f[v * 3 + k] = acc[k];
+#pragma unroll
+        for (int k = 0; k < 9; ++k) w[v * 9 + k] = acc[3 + k];
     }
-    f[v * 3 + 0] = fx;
-    f[v * 3 + 1] = fy;
-    f[v * 3 + 2] = fz;
-#pragma unroll
-    for (int k = 0; k < 9; ++k) w[v * 9 + k] = wv[k];
 }
 
 void launch_forces(int64_t n, const int* row_ptr, const int* rev, const float* gd,
                    const float4* geom, double* f_s, double* w_atom, cudaStream_t st) {
     if (n == 0) return;
-    forces_kernel<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(n, row_ptr, rev, gd, geom, f_s, w_atom);
+    forces_kernel<<<(unsigned)((n * FL + 127) / 128), 128, 0, st>>>(n, row_ptr, rev, gd, geom, f_s, w_atom);
 }
 
-// One CTA per structure: fixed-order FP64 sums of atom energies and virials
-// (per thread over a strided set of atoms, then a fixed shuffle tree per warp
-// and over the warps), so repeated evaluations give identical sums.
-constexpr int RS_THREADS = 1024;
+// FP64 sums of atom energies and virials per structure in a fixed order that
+// depends on the structure alone: a CTA per 512 atoms of a structure (two a thread,
+// a shuffle tree per warp, the warps in order), then a warp per structure over its
+// CTAs' partial sums.  One CTA per structure took 90 us for 24,000 atoms.
+constexpr int RS_ATOMS = 512, RS_THREADS = 256;
 
 __device__ __forceinline__ double warp_sum_d(double v) {
 #pragma unroll
@@ -429,15 +439,20 @@ __device__ __forceinline__ double warp_sum_d(double v) {
     return v;
 }
 
-__global__ void __launch_bounds__(RS_THREADS) reduce_structs_kernel(const int64_t* __restrict__ atom_off,
-                                                                    const double* __restrict__ e_atom,
-                                                                    const double* __restrict__ w_atom,
-                                                                    double* __restrict__ energy,
-                                                                    double* __restrict__ virial) {
-    const int s = blockIdx.x;
-    const int64_t a0 = atom_off[s], a1 = atom_off[s + 1];
+// first partial of structure s: structures never share one
+__device__ __forceinline__ int64_t partial_base(const int64_t* __restrict__ atom_off, int s) {
+    return atom_off[s] / RS_ATOMS + s;
+}
+
+__global__ void __launch_bounds__(RS_THREADS) reduce_partials_kernel(int s0,
+                                                                     const int64_t* __restrict__ atom_off,
+                                                                     const double* __restrict__ e_atom,
+                                                                     const double* __restrict__ w_atom,
+                                                                     double* __restrict__ partial) {
+    const int s = s0 + blockIdx.y;
+    const int64_t a0 = atom_off[s] + (int64_t)blockIdx.x * RS_ATOMS, a1 = min(atom_off[s + 1], a0 + RS_ATOMS);
+    if (a0 >= a1) return;
     double acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
-#pragma unroll 4
     for (int64_t v = a0 + threadIdx.x; v < a1; v += RS_THREADS) {
         acc[0] += e_atom[v];
 #pragma unroll
@@ -451,21 +466,42 @@ __global__ void __launch_bounds__(RS_THREADS) reduce_structs_kernel(const int64_
         if (lane == 0) red[warp][k] = w;
     }
     __syncthreads();
-    if (warp == 0) {
-#pragma unroll
-        for (int k = 0; k < 10; ++k) acc[k] = warp_sum_d(red[lane][k]);
-        if (lane == 0) {
-            if (energy) energy[s] = acc[0];
-            if (virial)
-                for (int k = 0; k < 9; ++k) virial[s * 9 + k] = acc[1 + k];
-        }
+    if (threadIdx.x < 10) {
+        double t = 0.0;
+        for (int i = 0; i < RS_THREADS / 32; ++i) t += red[i][threadIdx.x];
+        partial[(partial_base(atom_off, s) + blockIdx.x) * 10 + threadIdx.x] = t;
     }
 }
 
-void launch_reduce_structs(int32_t n_structs, const int64_t* atom_off, const double* e_atom,
-                           const double* w_atom, double* energy, double* virial, cudaStream_t st) {
+__global__ void reduce_structs_kernel(int n_structs, const int64_t* __restrict__ atom_off,
+                                      const double* __restrict__ partial, double* __restrict__ energy,
+                                      double* __restrict__ virial) {
+    const int s = (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5), lane = threadIdx.x & 31;
+    if (s >= n_structs) return;
+    const int64_t n = (atom_off[s + 1] - atom_off[s] + RS_ATOMS - 1) / RS_ATOMS, b = partial_base(atom_off, s);
+    double acc[10] = {0, 0, 0, 0, 0, 0, 0, 0, 0, 0};
+    for (int64_t i = lane; i < n; i += 32)
+#pragma unroll
+        for (int k = 0; k < 10; ++k) acc[k] += partial[(b + i) * 10 + k];
+#pragma unroll
+    for (int k = 0; k < 10; ++k) acc[k] = warp_sum_d(acc[k]);
+    if (lane == 0) {
+        if (energy) energy[s] = acc[0];
+        if (virial)
+            for (int k = 0; k < 9; ++k) virial[s * 9 + k] = acc[1 + k];
+    }
+}
+
+void launch_reduce_structs(int32_t n_structs, int64_t max_atoms, const int64_t* atom_off, const double* e_atom,
+                           const double* w_atom, double* partial, double* energy, double* virial, cudaStream_t st) {
     if (n_structs == 0) return;
-    reduce_structs_kernel<<<n_structs, RS_THREADS, 0, st>>>(atom_off, e_atom, w_atom, energy, virial);
+    const unsigned chunks = (unsigned)((max_atoms + RS_ATOMS - 1) / RS_ATOMS);
+    for (int32_t s0 = 0; chunks > 0 && s0 < n_structs; s0 += 65535) {    // grid.y is at most 65,535
+        const dim3 grid(chunks, (unsigned)std::min<int32_t>(65535, n_structs - s0));
+        reduce_partials_kernel<<<grid, RS_THREADS, 0, st>>>(s0, atom_off, e_atom, w_atom, partial);
+    }
+    reduce_structs_kernel<<<(unsigned)((n_structs * 32 + 127) / 128), 128, 0, st>>>(n_structs, atom_off, partial, energy,
+                                                                                    virial);
 }
 
 __global__ void scatter_forces_kernel(int64_t n, const int* __restrict__ perm,

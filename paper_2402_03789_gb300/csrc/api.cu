@@ -687,17 +687,22 @@ sevennet_status model_layer_backward_rest(sevennet_model* M, Workspace* ws, int 
     prof_end(&M->prof, PF_CONV_BWD, st, ev, t == 0 ? 1 : 2);
     count_launches(t == 0 ? 1 : 2);
     if (t == 0) return SEVENNET_OK;
-    GemmBatch a{}, c{};
+    GemmBatch a{};
     for (int l = 0; l < NL; ++l) {
         if (!L.in_mul[l]) continue;
-        a.p[a.n++] = GemmProb{ws->gx, L.lin1T[l], L.lin1Th[l], ws->gh, N, 2 * l + 1, L.in_mul[l], L.in_mul[l],
-                              L.x_dim, L.in_off[l], L.h_in_dim, L.in_off[l], 0};
-        if (L.y_mul[l])
-            c.p[c.n++] = GemmProb{ws->gy, L.scT[l], L.scTh[l], ws->gh, N, 2 * l + 1, L.y_mul[l], L.in_mul[l],
-                                  L.y_dim, L.y_off[l], L.h_in_dim, L.in_off[l], 1};
+        GemmProb p{ws->gx, L.lin1T[l], L.lin1Th[l], ws->gh, N, 2 * l + 1, L.in_mul[l], L.in_mul[l],
+                   L.x_dim, L.in_off[l], L.h_in_dim, L.in_off[l], 0};
+        if (L.y_mul[l]) {
+            p.K2 = L.y_mul[l];
+            p.lda2 = L.y_dim;
+            p.a_off2 = L.y_off[l];
+            p.A2 = ws->gy;
+            p.B2 = L.scT[l];
+            p.Bh2 = L.scTh[l];
+        }
+        a.p[a.n++] = p;
     }
     run_gemm(M, a, prec, st);
-    run_gemm(M, c, prec, st);
     return SEVENNET_OK;
 }
 

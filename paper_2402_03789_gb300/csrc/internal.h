@@ -335,6 +335,11 @@ struct GemmProb {
     int32_t R, K, N;           // K and N are multiples of 32 (every multiplicity is)
     int32_t lda, a_off, ldc, c_off;
     int32_t accumulate;        // 1: C += A B, 0: C = A B
+    // a second product added to the same rows (K2 = 0: none): C = A B + A2 B2
+    int32_t K2 = 0, lda2 = 0, a_off2 = 0;
+    const float* A2 = nullptr;
+    const float* B2 = nullptr;
+    const __nv_bfloat16* Bh2 = nullptr;
 };
 constexpr int MAX_GEMM_PROBS = 8;
 struct GemmBatch {

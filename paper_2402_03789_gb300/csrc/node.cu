@@ -22,53 +22,85 @@ __device__ __forceinline__ float dsilu_(float x) {
 }
 
 // ---------------------------------------------------------------- FP32 GEMM
-// 64 x 64 output tile, 256 threads, 4 x 4 per thread, K slices of 16.
-__global__ void __launch_bounds__(256)
-gemm_f32_kernel(const GemmBatch batch) {
+// TM x TN output tile, 4 x 4 per thread, K slices of 16 through a ring of four
+// stages filled by cp.async (a slice waited for its loads before: 17 us a launch
+// for cells of any size up to some hundred atoms).  Small problems take 32 x 32
+// tiles, which spread them over more SMs.  k runs in ascending order either way, so
+// a row's result does not depend on the batch it is in.
+constexpr int GK = 16, GST = 4;
+
+__device__ __forceinline__ void g_cp16(void* s, const void* g, bool valid) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(s)), "l"(g),
+                 "r"(valid ? 16 : 0) : "memory");
+}
+
+template <int TM, int TN>
+__global__ void __launch_bounds__(TM * TN / 16)
+gemm_f32_kernel(const __grid_constant__ GemmBatch batch) {
+    constexpr int NT = TM * TN / 16, NA = TM * GK / 4 / NT, NB = TN * GK / 4 / NT;
     const GemmProb& P = batch.p[blockIdx.z];
     const int64_t rows = P.n_atoms * P.R;
-    const int64_t r0 = (int64_t)blockIdx.x * 64;
-    const int n0 = blockIdx.y * 64;
+    const int64_t r0 = (int64_t)blockIdx.x * TM;
+    const int n0 = blockIdx.y * TN;
     if (r0 >= rows || n0 >= P.N) return;
-    __shared__ __align__(16) float sA[16][68];
-    __shared__ __align__(16) float sB[16][64];
+    __shared__ __align__(16) float sA[GST][TM][GK + 4];
+    __shared__ __align__(16) float sB[GST][GK][TN];
     const int t = threadIdx.x;
-    const int tr = t / 16, tc = t % 16;
+    const int tr = t / (TN / 4), tc = t % (TN / 4);
     float acc[4][4] = {};
-    // A loader: row = t / 4 (0..63), k quad = t % 4
-    const int lrow = t / 4, lkq = t % 4;
-    const int64_t arow = r0 + lrow;
-    const float* aptr = nullptr;
-    if (arow < rows) {
-        const int64_t v = arow / P.R;
-        const int mm = (int)(arow % P.R);
-        aptr = P.A + v * P.lda + P.a_off + (int64_t)mm * P.K;
+    // loaders: A row (t + i NT) / 4, k quad % 4; B row (t + i NT) / (TN / 4)
+    const float* aptr[NA][2];
+#pragma unroll
+    for (int i = 0; i < NA; ++i) {
+        const int64_t ar = r0 + (t + i * NT) / 4, v = (ar < rows ? ar : 0) / P.R;
+        const int mm = (int)((ar < rows ? ar : 0) % P.R);
+        aptr[i][0] = P.A + v * P.lda + P.a_off + (int64_t)mm * P.K;
+        aptr[i][1] = P.K2 ? P.A2 + v * P.lda2 + P.a_off2 + (int64_t)mm * P.K2 : nullptr;
     }
-    const int bk = t / 16, bc = t % 16;
-    for (int k0 = 0; k0 < P.K; k0 += 16) {
-        float4 av = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (aptr) av = *reinterpret_cast<const float4*>(aptr + k0 + 4 * lkq);
-        sA[4 * lkq + 0][lrow] = av.x;
-        sA[4 * lkq + 1][lrow] = av.y;
-        sA[4 * lkq + 2][lrow] = av.z;
-        sA[4 * lkq + 3][lrow] = av.w;
-        float4 bv = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (n0 + 4 * bc < P.N)
-            bv = __ldg(reinterpret_cast<const float4*>(P.B + (int64_t)(k0 + bk) * P.N + n0 + 4 * bc));
-        *reinterpret_cast<float4*>(&sB[bk][4 * bc]) = bv;
-        __syncthreads();
+    const int s1 = P.K / GK, slices = s1 + P.K2 / GK;
+    auto load = [&](int sl) {
+        const bool two = sl >= s1;
+        const int k0 = (two ? sl - s1 : sl) * GK, b = sl % GST;
+        const float* B = two ? P.B2 : P.B;
 #pragma unroll
-        for (int kk = 0; kk < 16; ++kk) {
-            const float4 a = *reinterpret_cast<const float4*>(&sA[kk][4 * tr]);
-            const float4 b = *reinterpret_cast<const float4*>(&sB[kk][4 * tc]);
-            const float aa[4] = {a.x, a.y, a.z, a.w};
-            const float bb[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-#pragma unroll
-                for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(aa[i], bb[j], acc[i][j]);
+        for (int i = 0; i < NA; ++i) {
+            const int q = t + i * NT;
+            g_cp16(&sA[b][q / 4][4 * (q % 4)], aptr[i][two] + k0 + 4 * (q % 4), r0 + q / 4 < rows);
         }
+#pragma unroll
+        for (int i = 0; i < NB; ++i) {
+            const int q = t + i * NT, kk = q / (TN / 4), col = n0 + 4 * (q % (TN / 4));
+            g_cp16(&sB[b][kk][4 * (q % (TN / 4))], B + (int64_t)(k0 + kk) * P.N + (col < P.N ? col : 0), col < P.N);
+        }
+    };
+#pragma unroll
+    for (int i = 0; i < GST - 1; ++i) {
+        if (i < slices) load(i);
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+    }
+    for (int sl = 0; sl < slices; ++sl) {
+        asm volatile("cp.async.wait_group %0;\n" ::"n"(GST - 2) : "memory");
         __syncthreads();
+        if (sl + GST - 1 < slices) load(sl + GST - 1);
+        asm volatile("cp.async.commit_group;\n" ::: "memory");
+        const int b = sl % GST;
+#pragma unroll
+        for (int k4 = 0; k4 < GK / 4; ++k4) {
+            float aa[4][4], bb[4][4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float4 q = *reinterpret_cast<const float4*>(&sA[b][4 * tr + i][4 * k4]);
+                aa[i][0] = q.x; aa[i][1] = q.y; aa[i][2] = q.z; aa[i][3] = q.w;
+                const float4 p = *reinterpret_cast<const float4*>(&sB[b][4 * k4 + i][4 * tc]);
+                bb[i][0] = p.x; bb[i][1] = p.y; bb[i][2] = p.z; bb[i][3] = p.w;
+            }
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) acc[i][j] = fmaf(aa[i][kk], bb[kk][j], acc[i][j]);
+        }
     }
     const int col = n0 + 4 * tc;
     if (col >= P.N) return;
@@ -118,8 +150,13 @@ __device__ __forceinline__ void mma_bf16_n(float* c, const uint32_t* a, const ui
 // k = kb + 8 tq + [0, 8), k step ks takes kb + 8 tq + 4 ks + [0, 4).  Its A
 // values are then one float4 per row and k step, and its B words (hi and lo)
 // one 16-byte load per n row and k block.  K and N are multiples of 32.
-__global__ void __launch_bounds__(256)
-gemm_bf16_kernel(const GemmBatch batch) {
+// PF: the next k block's operands are loaded before this one's MMAs (small
+// problems, one CTA or fewer per SM: their k blocks otherwise wait for memory one
+// after another); large problems hide it behind the other CTA of the SM instead.
+// DUAL: some problem has a second product.
+template <bool PF, bool DUAL>
+__global__ void __launch_bounds__(256, PF ? 1 : 2)
+gemm_bf16_kernel(const __grid_constant__ GemmBatch batch) {
     const GemmProb& P = batch.p[blockIdx.z];
     const int64_t rows = P.n_atoms * P.R;
     // N <= 32: the 8 warps stack as 8 x 1 over a 256 x 32 tile (the grid's extra
@@ -132,59 +169,85 @@ gemm_bf16_kernel(const GemmBatch batch) {
     const int wr = narrow ? warp : (warp & 3), wc = narrow ? 0 : (warp >> 2);
     const int nbase = n0 + wc * 32;
     if (nbase >= P.N) return;
-    auto rowptr = [&](int64_t r) -> const float* {
-        if (r >= rows) return nullptr;
-        const int64_t v = r / P.R;
-        const int mm = (int)(r % P.R);
-        return P.A + v * P.lda + P.a_off + (int64_t)mm * P.K;
-    };
     const float* pr[2][2];
-#pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
-#pragma unroll
-        for (int h = 0; h < 2; ++h) pr[mt][h] = rowptr(r0 + wr * 32 + mt * 16 + h * 8 + g);
     float c[2][4][4];
 #pragma unroll
     for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
         for (int j = 0; j < 4; ++j) c[mt][j][0] = c[mt][j][1] = c[mt][j][2] = c[mt][j][3] = 0.0f;
-    const int64_t lo_off = (int64_t)P.K * P.N;          // bf16 elements
     const float4 z4 = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int kb = 0; kb < P.K; kb += 32) {
+    struct Ops {
         uint4 bh[4], bl[4];
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const __nv_bfloat16* br = P.Bh + (int64_t)(nbase + j * 8 + g) * P.K + kb + 8 * tq;
-            bh[j] = __ldg(reinterpret_cast<const uint4*>(br));
-            bl[j] = __ldg(reinterpret_cast<const uint4*>(br + lo_off));
-        }
         float4 av[2][2][2];                                // [m tile][row half][k step]
+    };
+#pragma unroll 1
+    for (int seg = 0; seg < (DUAL ? 2 : 1); ++seg) {
+        const int K = seg ? P.K2 : P.K;
+        if (DUAL && K == 0) break;
+        const __nv_bfloat16* Bh = seg ? P.Bh2 : P.Bh;
+        const int64_t lo_off = (int64_t)K * P.N;           // bf16 elements
 #pragma unroll
         for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
+            for (int h = 0; h < 2; ++h) {
+                const int64_t r = r0 + wr * 32 + mt * 16 + h * 8 + g;
+                pr[mt][h] = r < rows ? (seg ? P.A2 + P.a_off2 : P.A + P.a_off) + r / P.R * (seg ? P.lda2 : P.lda) +
+                                           (int64_t)(int)(r % P.R) * K
+                                     : nullptr;
+            }
+        auto load = [&](int kb, Ops& o) {
 #pragma unroll
-                for (int ks = 0; ks < 2; ++ks)
-                    av[mt][h][ks] = pr[mt][h] ? *reinterpret_cast<const float4*>(pr[mt][h] + kb + 8 * tq + 4 * ks) : z4;
+            for (int j = 0; j < 4; ++j) {
+                const __nv_bfloat16* br = Bh + (int64_t)(nbase + j * 8 + g) * K + kb + 8 * tq;
+                o.bh[j] = __ldg(reinterpret_cast<const uint4*>(br));
+                o.bl[j] = __ldg(reinterpret_cast<const uint4*>(br + lo_off));
+            }
 #pragma unroll
-        for (int ks = 0; ks < 2; ++ks) {
+            for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-            for (int mt = 0; mt < 2; ++mt) {
-                uint32_t a[4], al[4];
-                split_bf16_n(av[mt][0][ks].x, av[mt][0][ks].y, a[0], al[0]);
-                split_bf16_n(av[mt][1][ks].x, av[mt][1][ks].y, a[1], al[1]);
-                split_bf16_n(av[mt][0][ks].z, av[mt][0][ks].w, a[2], al[2]);
-                split_bf16_n(av[mt][1][ks].z, av[mt][1][ks].w, a[3], al[3]);
+                for (int h = 0; h < 2; ++h)
 #pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    const uint32_t* wh = reinterpret_cast<const uint32_t*>(&bh[j]);
-                    const uint32_t* wl = reinterpret_cast<const uint32_t*>(&bl[j]);
-                    const uint32_t b[2] = {wh[2 * ks], wh[2 * ks + 1]};
-                    const uint32_t b2[2] = {wl[2 * ks], wl[2 * ks + 1]};
-                    mma_bf16_n(c[mt][j], a, b);
-                    if (GEMM_SPLIT_ACT) mma_bf16_n(c[mt][j], al, b);
-                    mma_bf16_n(c[mt][j], a, b2);
+                    for (int ks = 0; ks < 2; ++ks)
+                        o.av[mt][h][ks] = pr[mt][h] ? *reinterpret_cast<const float4*>(pr[mt][h] + kb + 8 * tq + 4 * ks) : z4;
+        };
+        auto mul = [&](const Ops& o) {
+#pragma unroll
+            for (int ks = 0; ks < 2; ++ks) {
+#pragma unroll
+                for (int mt = 0; mt < 2; ++mt) {
+                    uint32_t a[4], al[4];
+                    split_bf16_n(o.av[mt][0][ks].x, o.av[mt][0][ks].y, a[0], al[0]);
+                    split_bf16_n(o.av[mt][1][ks].x, o.av[mt][1][ks].y, a[1], al[1]);
+                    split_bf16_n(o.av[mt][0][ks].z, o.av[mt][0][ks].w, a[2], al[2]);
+                    split_bf16_n(o.av[mt][1][ks].z, o.av[mt][1][ks].w, a[3], al[3]);
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const uint32_t* wh = reinterpret_cast<const uint32_t*>(&o.bh[j]);
+                        const uint32_t* wl = reinterpret_cast<const uint32_t*>(&o.bl[j]);
+                        const uint32_t b[2] = {wh[2 * ks], wh[2 * ks + 1]};
+                        const uint32_t b2[2] = {wl[2 * ks], wl[2 * ks + 1]};
+                        mma_bf16_n(c[mt][j], a, b);
+                        if (GEMM_SPLIT_ACT) mma_bf16_n(c[mt][j], al, b);
+                        mma_bf16_n(c[mt][j], a, b2);
+                    }
                 }
+            }
+        };
+        if constexpr (PF) {
+            Ops o0, o1;
+            load(0, o0);
+            for (int kb = 0; kb < K; kb += 64) {
+                if (kb + 32 < K) load(kb + 32, o1);
+                mul(o0);
+                if (kb + 32 >= K) break;
+                if (kb + 64 < K) load(kb + 64, o0);
+                mul(o1);
+            }
+        } else {
+            for (int kb = 0; kb < K; kb += 32) {
+                Ops o;
+                load(kb, o);
+                mul(o);
             }
         }
     }
@@ -220,12 +283,26 @@ void launch_gemm(const GemmBatch& b, sevennet_precision prec, cudaStream_t st) {
         max_n = std::max(max_n, b.p[i].N);
     }
     if (max_rows == 0) return;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const int64_t sms = num_sms(dev);
     if (prec == SEVENNET_BF16) {
         const dim3 grid((unsigned)((max_rows + 127) / 128), (unsigned)((max_n + 63) / 64), (unsigned)b.n);
-        gemm_bf16_kernel<<<grid, 256, 0, st>>>(b);
+        bool dual = false;
+        for (int i = 0; i < b.n; ++i) dual = dual || b.p[i].K2 > 0;
+        const bool pf = (int64_t)grid.x * grid.y * grid.z <= sms;
+        if (pf && dual) gemm_bf16_kernel<true, true><<<grid, 256, 0, st>>>(b);
+        else if (pf) gemm_bf16_kernel<true, false><<<grid, 256, 0, st>>>(b);
+        else if (dual) gemm_bf16_kernel<false, true><<<grid, 256, 0, st>>>(b);
+        else gemm_bf16_kernel<false, false><<<grid, 256, 0, st>>>(b);
     } else {
         const dim3 grid((unsigned)((max_rows + 63) / 64), (unsigned)((max_n + 63) / 64), (unsigned)b.n);
-        gemm_f32_kernel<<<grid, 256, 0, st>>>(b);
+        if ((int64_t)grid.x * grid.y * grid.z < 2 * sms) {
+            const dim3 small((unsigned)((max_rows + 31) / 32), (unsigned)((max_n + 31) / 32), (unsigned)b.n);
+            gemm_f32_kernel<32, 32><<<small, 64, 0, st>>>(b);
+        } else {
+            gemm_f32_kernel<64, 64><<<grid, 256, 0, st>>>(b);
+        }
     }
 }
 

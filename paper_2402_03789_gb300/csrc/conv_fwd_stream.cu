@@ -548,25 +548,14 @@ __global__ void st_pack_kernel(const StRows R, int tiles, const float* __restric
 // by its helpers' copies (about 110 cycles of issue each, four helpers) if those
 // take longer.  ok = 0 where a type does not fit shared memory: the block then
 // keeps the chunked kernels.
-sevennet_status st_plan_build(sevennet_model* M, LayerDev& L) {
-    const ConvDesc& D = L.conv;
-    L.st[0].ok = L.st[1].ok = 0;
-    if (D.H != 64) return SEVENNET_OK;
-    struct U { int l1, set, g; };
-    std::vector<U> units;
-    for (int l1 = D.lmax; l1 >= 0; --l1) {
-        const StSets S = st_sets(l1, D.lmax, D.kind);
-        if (S.n > ST_MAX_SETS) return SEVENNET_OK;
-        if (!D.mul_in[l1]) continue;
-        for (int g = 0; g < D.mul_in[l1] / 32; ++g)
-            for (int j = 0; j < S.n; ++j) units.push_back({l1, j, g});
-    }
+struct StU { int l1, set, g; };
+
+static void st_plan_types(const ConvDesc& D, const std::vector<StU>& units, int sms, StPlan (&plan)[2]) {
+    using U = StU;
     const int n_types = ((int)units.size() + 3) / 4;
-    if (n_types < 1 || n_types > ST_MAX_TYPES) return SEVENNET_OK;
-    const int sms = num_sms(M->device);
-    if (sms < n_types) return SEVENNET_OK;
     for (int bf = 0; bf < 2; ++bf) {
-        StPlan& P = L.st[bf];
+        StPlan& P = plan[bf];
+        P = StPlan{};
         P.n_types = n_types;
         std::vector<int> cost(n_types, 0);
         int max_fixed = 0;
@@ -588,7 +577,11 @@ sevennet_status st_plan_build(sevennet_model* M, LayerDev& L) {
                     T.seg_floats[k] = 32;
                 }
                 const int g0 = (T.seg_src[k] - D.x_off[u.l1]) / 32;
-                T.seg_floats[k] = std::max(T.seg_floats[k], 32 * (u.g - g0 + 1));
+                if (u.g < g0) {
+                    T.seg_src[k] -= 32 * (g0 - u.g);
+                    T.seg_floats[k] += 32 * (g0 - u.g);
+                }
+                T.seg_floats[k] = std::max(T.seg_floats[k], 32 * (u.g - std::min(g0, u.g) + 1));
             }
             for (int k = 0; k < T.n_seg; ++k) { T.seg_dst[k] = row; row += T.seg_n[k] * T.seg_floats[k]; }
             T.row_floats = row;
@@ -652,6 +645,31 @@ sevennet_status st_plan_build(sevennet_model* M, LayerDev& L) {
         P.n_cta = at;
         P.ok = 1;
     }
+}
+
+sevennet_status st_plan_build(sevennet_model* M, LayerDev& L) {
+    using U = StU;
+    const ConvDesc& D = L.conv;
+    L.st[0].ok = L.st[1].ok = 0;
+    if (D.H != 64) return SEVENNET_OK;
+    const int sms = num_sms(M->device);
+    std::vector<StU> units;
+    // a type's four units: first the channel groups of a set, so that a type reads
+    // whole irrep blocks (one copy a row; a part of a block takes one per component);
+    // where such rows are too wide, first the sets of a group
+    for (int by_group = 0; by_group < 2 && !(L.st[0].ok && L.st[1].ok); ++by_group) {
+        units.clear();
+        for (int l1 = D.lmax; l1 >= 0; --l1) {
+            const int ns = st_sets(l1, D.lmax, D.kind).n, ng = D.mul_in[l1] / 32;
+            if (ns > ST_MAX_SETS) return SEVENNET_OK;
+            for (int k = 0; k < ns * ng; ++k)
+                units.push_back(by_group ? StU{l1, k % ns, k / ns} : StU{l1, k / ng, k % ng});
+        }
+        const int n_types = ((int)units.size() + 3) / 4;
+        if (n_types < 1 || n_types > ST_MAX_TYPES || sms < n_types) return SEVENNET_OK;
+        st_plan_types(D, units, sms, L.st);
+    }
+    const int n_types = L.st[0].n_types;
     // W3 as the A operand: row 32 r + lane of tile i = path i of unit r; three BF16
     // terms, of which the BF16 path reads the first
     for (int t = 0; t < n_types; ++t) {

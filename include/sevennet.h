@@ -23,7 +23,9 @@
  *                  returned by sevennet_last_error().  No call aborts or traps.
  *   Threads      : one model may be used from one thread at a time, except the
  *                  server API, which is thread-safe.
- *   Precision    : SEVENNET_FP32 computes every step in FP32 (FFMA, no TF32);
+ *   Precision    : SEVENNET_FP32 computes every step to FP32 accuracy (FP32 units,
+ *                  and on tensor cores the radial-MLP products with operands
+ *                  as sums of three BF16 terms, 24 mantissa bits, no TF32);
  *                  SEVENNET_BF16 runs the radial-MLP and node-linear matrix
  *                  products on tensor cores with BF16 operands and FP32
  *                  accumulation.  Distances and spherical harmonics are FP32;

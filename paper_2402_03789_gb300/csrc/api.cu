@@ -296,12 +296,6 @@ static std::vector<float> scaled(const double* w, int rows, int cols, double s, 
     return o;
 }
 
-static std::vector<__nv_bfloat16> to_bf16(const std::vector<float>& f) {
-    std::vector<__nv_bfloat16> o(f.size());
-    for (size_t i = 0; i < f.size(); ++i) o[i] = __float2bfloat16_rn(f[i]);
-    return o;
-}
-
 // hi = bf16(w) followed by lo = bf16(w - hi): two BF16 terms that carry w to
 // about 16 mantissa bits (used where a tensor-core product takes both).
 static std::vector<__nv_bfloat16> to_bf16_pair(const std::vector<float>& f) {
@@ -312,6 +306,32 @@ static std::vector<__nv_bfloat16> to_bf16_pair(const std::vector<float>& f) {
         o[f.size() + i] = __float2bfloat16_rn(f[i] - __bfloat162float(h));
     }
     return o;
+}
+
+// Three BF16 terms of n FP32 values (see conv_common.cuh), one array after another.
+__global__ void terms_kernel(int64_t n, const float* __restrict__ w, __nv_bfloat16* __restrict__ out) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    float v = w[i];
+    for (int z = 0; z < 3; ++z) {
+        const __nv_bfloat16 h = __float2bfloat16_rn(v);
+        out[z * n + i] = h;
+        v -= __bfloat162float(h);
+    }
+}
+
+static sevennet_status dev_terms(sevennet_model* M, const float* w, size_t n, __nv_bfloat16** out) {
+    void* p = nullptr;
+    if (cudaMalloc(&p, 3 * n * sizeof(__nv_bfloat16)) != cudaSuccess) {
+        cudaGetLastError();
+        set_error("cudaMalloc of %zu bytes failed", 3 * n * sizeof(__nv_bfloat16));
+        return SEVENNET_ENOMEM;
+    }
+    M->allocations.push_back(p);
+    terms_kernel<<<(unsigned)((n + 255) / 256), 256>>>((int64_t)n, w, static_cast<__nv_bfloat16*>(p));
+    SN_CUDA(cudaGetLastError());
+    *out = static_cast<__nv_bfloat16*>(p);
+    return SEVENNET_OK;
 }
 
 static sevennet_status upload_linear(sevennet_model* M, const double* w, int rows, int cols, double s,
@@ -967,16 +987,17 @@ sevennet_status sevennet_create_model(const sevennet_model_config* cfg, const do
             const double s2 = 1.0 / std::sqrt((double)H) / cfg->avg_num_neigh;
             auto w2 = scaled(weights + e2->off, H, D.W, s2, false);
             auto w2T = scaled(weights + e2->off, H, D.W, s2, true);
-            if ((s = dev_upload(M, w0, &L.mlp0))) return fail(s);
-            if ((s = dev_upload(M, w1, &L.mlp1))) return fail(s);
             auto w1T = scaled(weights + e1->off, H, H, 1.0 / std::sqrt((double)H), true);
+            float *w1_dev = nullptr, *w2_dev = nullptr;
+            if ((s = dev_upload(M, w0, &L.mlp0))) return fail(s);
+            if ((s = dev_upload(M, w1, &w1_dev))) return fail(s);
             if ((s = dev_upload(M, w1T, &L.mlp1T))) return fail(s);
-            if ((s = dev_upload(M, to_bf16_pair(w1), &L.mlp1h))) return fail(s);     // [k][j] hi, lo
-            if ((s = dev_upload(M, to_bf16_pair(w1T), &L.mlp1Th))) return fail(s);   // [j][k] hi, lo
-            if ((s = dev_upload(M, w2, &L.mlp2))) return fail(s);
+            if ((s = dev_upload(M, w2, &w2_dev))) return fail(s);
             if ((s = dev_upload(M, w2T, &L.mlp2T))) return fail(s);
-            if ((s = dev_upload(M, to_bf16(w2T), &L.mlp2h))) return fail(s);   // [W][H]
-            if ((s = dev_upload(M, to_bf16(w2), &L.mlp2Th))) return fail(s);   // [H][W]
+            if ((s = dev_terms(M, w1_dev, w1.size(), &L.mlp1h))) return fail(s);     // [k][j]
+            if ((s = dev_terms(M, L.mlp1T, w1.size(), &L.mlp1Th))) return fail(s);   // [j][k]
+            if ((s = dev_terms(M, L.mlp2T, w2.size(), &L.mlp2h))) return fail(s);    // [W][H]
+            if ((s = dev_terms(M, w2_dev, w2.size(), &L.mlp2Th))) return fail(s);    // [H][W]
             if ((s = radial_pack(M, L))) return fail(s);
             if ((s = st_plan_build(M, L))) return fail(s);
         }
@@ -985,6 +1006,10 @@ sevennet_status sevennet_create_model(const sevennet_model_config* cfg, const do
     if (!s) s = st_configure(M->lmax);
     if (s) return fail(s);
     M->h2_bytes = st_h2_bytes(M);
+    if (cudaStreamSynchronize(nullptr) != cudaSuccess) {        // the weight preparation kernels
+        set_error("weight preparation failed: %s", cudaGetErrorString(cudaGetLastError()));
+        return fail(SEVENNET_ECUDA);
+    }
     if (cudaStreamCreateWithFlags(&M->stream, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
         set_error("cudaStreamCreate failed");

@@ -293,9 +293,7 @@ __device__ __forceinline__ void tp_bwd_chunk_pair(const ConvDesc& D, int ne, con
 // units (read on the device).
 template <int H, bool BF, int LMAX, bool PAIR>
 __global__ void __launch_bounds__(CONV_THREADS, conv_ctas_per_sm(LMAX))
-conv_bwd_kernel(const ConvDesc D, const float* __restrict__ W1, const float* __restrict__ W2,
-                const float* __restrict__ W2T, const float* __restrict__ W3, const float* __restrict__ W3T,
-                const __nv_bfloat16* __restrict__ W3T_h, const __nv_bfloat16* __restrict__ W3_h,
+conv_bwd_kernel(const ConvDesc D, const float* __restrict__ W1, const __nv_bfloat16* __restrict__ W3T_h, const __nv_bfloat16* __restrict__ W3_h,
                 const __nv_bfloat16* __restrict__ W2T_h, const __nv_bfloat16* __restrict__ W2_h,
                 int tile_units, const int* __restrict__ count, const int* __restrict__ dst,
                 const int* __restrict__ src, const float4* __restrict__ geom, const int* __restrict__ eidx,
@@ -351,7 +349,7 @@ conv_bwd_kernel(const ConvDesc D, const float* __restrict__ W1, const float* __r
             cur.geom = s_ngeo[t];
             if constexpr (PAIR) s_ecur[t] = s_ne[t];      // published by the prologue's barrier
         }
-        chunk_prologue<H, BF, LMAX>(D, L, smem, c0, ne, cur, W2, W2T_h);
+        chunk_prologue<H, BF, LMAX>(D, L, smem, c0, ne, cur, W2T_h);
         stage(c0 + EC);        // lands by the wait before phase G
         // dE/dd of the blocks done so far, copied to shared memory for phase G
         if (t < 3 * ne) {
@@ -359,8 +357,7 @@ conv_bwd_kernel(const ConvDesc D, const float* __restrict__ W1, const float* __r
             else cp_async4(s_gdp + t, gd + (size_t)c0 * 3 + t);
         }
         cp_async_commit();
-        if constexpr (BF) chunk_w_gemm_bf16<H, false>(D, L, smem, W3T_h);
-        else chunk_w_gemm_f32<H>(D, L, smem, W3);
+        chunk_w_gemm<H, BF ? 1 : 3, false>(D, L, smem, W3T_h);
         // E: per-edge (or per-pair) adjoint of the tensor product (path lists fixed per
         // block kind); the H = 32 kernels (small models) take one channel per lane
         constexpr int MAXC = H == 64 ? 2 : 1;
@@ -380,22 +377,22 @@ conv_bwd_kernel(const ConvDesc D, const float* __restrict__ W1, const float* __r
             }
         }
         // F: dE/dH2 = dE/dw @ W3^T
-        if constexpr (BF) chunk_gw_gemm_bf16<H, PAIR>(D, L, smem, W3_h);
-        else chunk_gw_gemm_f32<H>(D, L, smem, W3T);
+        chunk_gw_gemm<H, BF ? (PAIR ? 2 : 1) : 3, BF ? 1 : 3>(D, L, smem, W3_h);
         // MLP adjoint: gA2 = gH2 * silu'(A2); gH1 = gA2 @ W2^T; gA1 = gH1 * silu'(A1); gB = gA1 @ W1^T
         float* s_gH = smem + L.gH;
         float* s_A1 = smem + L.A1;
         float* s_A2 = smem + L.A2;
         for (int i = t; i < H * EC; i += CONV_THREADS) s_gH[i] *= dsiluf_(s_A2[i]);
         __syncthreads();
-        if constexpr (BF) {   // gA1 = (gA2 @ W2^T) * silu'(A1) on tensor cores, stored over A2
+        {   // gA1 = (gA2 @ W2^T) * silu'(A1), stored over A2
+            constexpr int AT = BF ? (PAIR ? 2 : 1) : 3, BT = BF ? 2 : 3;
             const int lane = t & 31, g = lane >> 2, tq = lane & 3;
             float c[4] = {0.f, 0.f, 0.f, 0.f};
             const int nt = warp;
             if (nt < H / 8) {
-                HiddenB<H> hb;
-                hidden_load<H>(W2_h, nt, hb);
-                hidden_mma<H, PAIR>(s_gH, hb, c);
+                HiddenB<H, BT> hb;
+                hidden_load<H, BT>(W2_h, nt, hb);
+                hidden_mma<H, AT, BT>(s_gH, hb, c);
             }
             __syncthreads();       // every read of A2 (the silu' above) is done
             if (nt < H / 8) {
@@ -403,33 +400,6 @@ conv_bwd_kernel(const ConvDesc D, const float* __restrict__ W1, const float* __r
                 const int o[4] = {hk<H>(k, g), hk<H>(k + 1, g), hk<H>(k, g + 8), hk<H>(k + 1, g + 8)};
 #pragma unroll
                 for (int q = 0; q < 4; ++q) s_A2[o[q]] = c[q] * dsiluf_(s_A1[o[q]]);
-            }
-        } else {   // gA1 = (gA2 @ W2^T) * silu'(A1), stored over A2; W2T[j][k] = W2[k][j]
-            float ga[(H / 4) * EC / CONV_THREADS > 0 ? (H / 4) * EC / CONV_THREADS : 1][4];
-            int nq = 0;
-            for (int idx = t; idx < (H / 4) * EC; idx += CONV_THREADS, ++nq) {
-                const int kq = idx / EC, e = idx % EC;
-                float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll 8
-                for (int j = 0; j < H; ++j) {
-                    const float4 b = __ldg(reinterpret_cast<const float4*>(W2T + j * H) + kq);
-                    const float a = s_gH[hk<H>(j, e)];
-                    a0 = fmaf(a, b.x, a0);
-                    a1 = fmaf(a, b.y, a1);
-                    a2 = fmaf(a, b.z, a2);
-                    a3 = fmaf(a, b.w, a3);
-                }
-                ga[nq][0] = a0; ga[nq][1] = a1; ga[nq][2] = a2; ga[nq][3] = a3;
-            }
-            __syncthreads();       // every read of A2 (the silu' above) is done
-            nq = 0;
-            for (int idx = t; idx < (H / 4) * EC; idx += CONV_THREADS, ++nq) {
-                const int kq = idx / EC, e = idx % EC;
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const int o = hk<H>(4 * kq + q, e);
-                    s_A2[o] = ga[nq][q] * dsiluf_(s_A1[o]);
-                }
             }
         }
         __syncthreads();
@@ -534,7 +504,7 @@ void conv_bwd_dispatch(const LayerDev& L, int H, bool bf, int64_t bound, const i
     const int grid = (int)std::max<int64_t>(1, (bound + tile - 1) / tile);
     const size_t sm = smem_bytes(L.conv, H, true, bf);
 #define SN_LB(HH, BB, LL) conv_bwd_kernel<HH, BB, LL, PAIR><<<grid, CONV_THREADS, sm, st>>>(           \
-        L.conv, L.mlp0, L.mlp1, L.mlp1T, L.mlp2, L.mlp2T, L.mlp2h, L.mlp2Th, L.mlp1Th, L.mlp1h,       \
+        L.conv, L.mlp0, L.mlp2h, L.mlp2Th, L.mlp1Th, L.mlp1h,       \
         tile, count, dst, src, geom, eidx, x, gm, gxq, gd)
     if (H == 64) {
         if (bf) { if (lm == 3) SN_LB(64, true, 3); else if (lm == 2) SN_LB(64, true, 2); else SN_LB(64, true, 1); }

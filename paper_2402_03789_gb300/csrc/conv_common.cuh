@@ -16,9 +16,9 @@
 // count) and walks its edges, sorted by receiver, in chunks of EC edges.
 // Adjoint: one CTA per tile of up to 4 chunks, tiles in edge order.  Per chunk:
 //   A  geometry: r, unit vector, Y (l <= 2), Bessel basis x envelope  (FP32)
-//   B  radial MLP hidden layers                                      (FFMA)
+//   B  radial MLP hidden layers
 //   C  G matrices of every path for every edge of the chunk
-//   D  w = H2 @ W3 for all W columns into shared memory              (FFMA)
+//   D  w = H2 @ W3 for all W columns into shared memory   (tensor cores)
 //   E  forward: each warp owns 32-channel groups of paths and walks the edges,
 //      keeping the running sum of the current receiver in registers and writing
 //      it once when the receiver changes (segmented sum, no atomics);
@@ -31,10 +31,6 @@
 #include <utility>
 
 namespace sn {
-
-constexpr int KS = 8;         // k-slice of the W3 staging in phase D
-constexpr int DCOLS = 512;    // columns per pass of phase D
-constexpr int CS = 32;        // column slice of phase F (adjoint W3 product)
 
 struct ConvSmem {
     int w, stage, A1, A2, H2, gH, G, Y, B, gY, src, dst, first, W1, geo, gdp, total;
@@ -63,20 +59,17 @@ __device__ __forceinline__ void hk_inv(int i, int& k, int& e) {
     e = p & 15;
 }
 
-// The staging region holds H1 and dE/dbasis on both paths, and the W3 slices of
-// the FP32 phases D and F on the FP32 path only.  dE/dH2 (adjoint) reuses H2,
-// which is dead once phase D has run.  The BF16 kernels stay under 97 KB so two
-// CTAs leave about 60 KB of each SM's 256 KB to the L1 cache.
+// The staging region holds H1 and dE/dbasis.  dE/dH2 (adjoint) reuses H2, which is
+// dead once phase D has run.  The BF16 kernels stay under 97 KB so two CTAs leave
+// about 60 KB of each SM's 256 KB to the L1 cache.
 __host__ __device__ inline ConvSmem conv_smem_layout(int Wpad, int WpadB, int H, int nG, int ys, bool bwd, bool bf) {
     ConvSmem s;
     int o = 0;
-    const int stage_bf = H * EC > MAX_NB * EC ? H * EC : MAX_NB * EC;
-    const int stage_f32 = KS * DCOLS > 2 * CS * 64 ? KS * DCOLS : 2 * CS * 64;
-    // [EC][row stride]: BF16 in the BF16 forward; the BF16 adjoint also keeps three
+    // [EC][row stride]: BF16 in the BF16 forward; the adjoint also keeps three
     // [H][EC] partials of phase F there
-    const int w_bwd_bf = EC * Wpad > 3 * H * EC ? EC * Wpad : 3 * H * EC;
-    s.w = o;     o += (bf && !bwd) ? EC * WpadB / 2 : (bf ? w_bwd_bf : EC * Wpad);
-    s.stage = o; o += bf ? stage_bf : (stage_f32 > stage_bf ? stage_f32 : stage_bf);
+    const int w_bwd = EC * Wpad > 3 * H * EC ? EC * Wpad : 3 * H * EC;
+    s.w = o;     o += bwd ? w_bwd : (bf ? EC * WpadB / 2 : EC * Wpad);
+    s.stage = o; o += H * EC > MAX_NB * EC ? H * EC : MAX_NB * EC;
     s.A1 = o;    o += H * EC;
     s.A2 = o;    o += H * EC;
     s.H2 = o;    o += H * EC;
@@ -223,7 +216,7 @@ struct BlockPaths {
     static constexpr int begin = path_begin(L1, LMAX, KIND);
 };
 
-// ---- BF16 tensor-core variants of phases D and F (mma.sync m16n8k16, FP32 accumulate)
+// ---- phases D and F on tensor cores (mma.sync m16n8k16, FP32 accumulate)
 // The per-edge weight tile holds BF16 values in the BF16 forward kernel and
 // FP32 values otherwise (the adjoint keeps dE/dw in FP32 beside w).
 template <bool BF>
@@ -250,10 +243,25 @@ __device__ __forceinline__ float4 unpack_bf16x4(uint32_t a, uint32_t b) {
                        __uint_as_float(b & 0xffff0000u));
 }
 
-// Activations enter the tensor cores as one BF16 value (round to nearest).  W3
-// is one BF16 value too; the hidden-layer weights W2 are a hi + lo BF16 pair
-// (two MMAs), which keeps the virial error of the BF16 path near that of its
-// forces (a single BF16 W2 raised it about fivefold).
+// Operands enter the tensor cores as sums of BF16 terms, each the BF16 value
+// nearest to what the terms before it leave.  BF16 path: one term for the
+// activations and W3, two for the hidden-layer weights W2 (a single BF16 W2 raised
+// the virial error fivefold).  FP32 path: three terms of everything, 24 mantissa
+// bits.  Products of terms i and j are taken while i + j is below the larger number
+// of terms (six for three terms; those left out are below 2^-24).  The tensor cores
+// truncate where an FP32 unit rounds, so the FP32 path keeps their chains short: the
+// leading products of a k step start from zero and are added by FADD, the small
+// ones run in a chain of their own (in one chain dE/dd was 2.0e-6 off in FP32,
+// twice the error of FFMA sums).
+template <int NT>
+__device__ __forceinline__ void bf16_terms(float x, float y, uint32_t (&t)[NT]) {
+#pragma unroll
+    for (int z = 0; z < NT; ++z) {
+        t[z] = pack_bf16(x, y);
+        x -= __uint_as_float(t[z] << 16);
+        y -= __uint_as_float(t[z] & 0xffff0000u);
+    }
+}
 
 __device__ __forceinline__ void mma_bf16(float* c, const uint32_t* a, const uint32_t* b) {
     asm volatile(
@@ -269,49 +277,68 @@ __device__ __forceinline__ void mma_bf16(float* c, const uint32_t* a, const uint
 // operand two contiguous 16-byte loads; k step ks then uses words
 // w0 = tq * 2 KSN + 2 ks (first half of the fragment) and w0 + 1 (second half).
 
-// Phase D (BF16): w[e][c] = sum_k H2[k][e] W3[k][c]; B operand W3T [W][H] (bf16).
-// Each warp loads the B fragments of four n tiles at once.
-template <int H, bool BFT>
-__device__ __forceinline__ void chunk_w_gemm_bf16(const ConvDesc& D, const ConvSmem& L, float* smem,
-                                                  const __nv_bfloat16* __restrict__ W3T) {
+// Phase D: w[e][c] = sum_k H2[k][e] W3[k][c]; B operand W3T, NT terms of [W][H].
+// Each warp loads the B fragments of BATCH n tiles at once.  FP32: FFMA took 61,440
+// multiply-adds an edge on FP32 lanes, more than half of the FP32 adjoint's time.
+template <int H, int NT, bool BFT>
+__device__ __forceinline__ void chunk_w_gemm(const ConvDesc& D, const ConvSmem& L, float* smem,
+                                             const __nv_bfloat16* __restrict__ W3T) {
     constexpr int KSN = H / 16;                // k steps (4 or 2)
-    constexpr int NV = KSN / 2;                // 16-byte loads per lane and n tile
-    constexpr int BATCH = 4;
+    constexpr int NV = KSN / 2;                // 16-byte loads per lane, n tile and term
+    constexpr int BATCH = NT == 1 ? 4 : 1;
     static_assert(EC == 16, "one m tile of edges");
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, g = lane >> 2, tq = lane & 3;
     const float* s_H2 = smem + L.H2;
-    uint32_t af[KSN][4];
+    uint32_t af[NT][KSN][4];
 #pragma unroll
-    for (int ks = 0; ks < KSN; ++ks) {
-        const int k0 = 2 * (tq * 2 * KSN + 2 * ks), k1 = k0 + 2;
-        af[ks][0] = pack_bf16(s_H2[hk<H>(k0, g)], s_H2[hk<H>(k0 + 1, g)]);
-        af[ks][1] = pack_bf16(s_H2[hk<H>(k0, g + 8)], s_H2[hk<H>(k0 + 1, g + 8)]);
-        af[ks][2] = pack_bf16(s_H2[hk<H>(k1, g)], s_H2[hk<H>(k1 + 1, g)]);
-        af[ks][3] = pack_bf16(s_H2[hk<H>(k1, g + 8)], s_H2[hk<H>(k1 + 1, g + 8)]);
-    }
+    for (int ks = 0; ks < KSN; ++ks)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int k = 2 * (tq * 2 * KSN + 2 * ks) + 2 * (q >> 1), e = g + 8 * (q & 1);
+            uint32_t tt[NT];
+            bf16_terms<NT>(s_H2[hk<H>(k, e)], s_H2[hk<H>(k + 1, e)], tt);
+#pragma unroll
+            for (int z = 0; z < NT; ++z) af[z][ks][q] = tt[z];
+        }
     const int ntiles = D.W / 8;
+    const size_t term = (size_t)D.W * H;
     for (int nb = warp; nb < ntiles; nb += BATCH * CONV_WARPS) {
-        uint4 bv[BATCH][NV];
+        uint4 bv[BATCH][NT][NV];
 #pragma unroll
         for (int j = 0; j < BATCH; ++j) {
             const int nt = nb + j * CONV_WARPS;
             if (nt < ntiles) {
-                const uint4* row = reinterpret_cast<const uint4*>(W3T + (size_t)(nt * 8 + g) * H);
 #pragma unroll
-                for (int v = 0; v < NV; ++v) bv[j][v] = __ldg(row + tq * NV + v);
+                for (int z = 0; z < NT; ++z) {
+                    const uint4* row = reinterpret_cast<const uint4*>(W3T + z * term + (size_t)(nt * 8 + g) * H);
+#pragma unroll
+                    for (int v = 0; v < NV; ++v) bv[j][z][v] = __ldg(row + tq * NV + v);
+                }
             }
         }
 #pragma unroll
         for (int j = 0; j < BATCH; ++j) {
             const int nt = nb + j * CONV_WARPS;
             if (nt >= ntiles) break;
-            const uint32_t* bw = reinterpret_cast<const uint32_t*>(bv[j]);
-            float c[4] = {0.f, 0.f, 0.f, 0.f};
+            float c[4] = {}, cs[4] = {};       // leading and small products
 #pragma unroll
             for (int ks = 0; ks < KSN; ++ks) {
-                const uint32_t b[2] = {bw[2 * ks], bw[2 * ks + 1]};
-                mma_bf16(c, af[ks], b);
+                float ct[4] = {};
+#pragma unroll
+                for (int o = NT - 1; o >= 0; --o)
+#pragma unroll
+                    for (int z = 0; z <= o; ++z) {
+                        const uint32_t* bw = reinterpret_cast<const uint32_t*>(bv[j][o - z]);
+                        const uint32_t b[2] = {bw[2 * ks], bw[2 * ks + 1]};
+                        mma_bf16(o > 0 ? cs : (NT == 3 ? ct : c), af[z][ks], b);
+                    }
+                if constexpr (NT == 3) {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) c[q] += ct[q];
+                }
             }
+#pragma unroll
+            for (int q = 0; q < 4; ++q) c[q] += cs[q];
             const int col = nt * 8 + 2 * tq;
             if constexpr (BFT) {         // BF16 tile [EC][WpadB]
                 __nv_bfloat16* s_w = reinterpret_cast<__nv_bfloat16*>(smem + L.w);
@@ -328,20 +355,20 @@ __device__ __forceinline__ void chunk_w_gemm_bf16(const ConvDesc& D, const ConvS
     __syncthreads();
 }
 
-// Phase F (BF16): gH2[k][e] = sum_c gw[e][c] W3[k][c]; B operand W3 [H][W] (bf16).
+// Phase F: gH2[k][e] = sum_c gw[e][c] W3[c][k]; A operand dE/dw in AT terms, B
+// operand W3 in BT terms of [H][W].
 // K (the W columns, in blocks of 32) is split between four groups of two warps;
 // within a group each warp owns H/16 n tiles of 8 hidden units for the group's
 // whole K range, so every output has one writer per group.  Group 0 writes
 // dE/dH2; groups 1-3 write partials into the dE/dw tile once every warp is done
-// reading it (the BF16 adjoint's tile holds at least three [H][EC] partials),
+// reading it (the adjoint's tile holds at least three [H][EC] partials),
 // and the partials are added in group order, so the result does not depend on
 // the warps' timing.
-// SPLIT: dE/dw enters as a hi + lo BF16 pair (two MMAs per n tile), which keeps
-// about 16 bits of it (the pair kernel's dE/dw is the sum of two directions).
-template <int H, bool SPLIT = false>
-__device__ __forceinline__ void chunk_gw_gemm_bf16(const ConvDesc& D, const ConvSmem& L, float* smem,
-                                                   const __nv_bfloat16* __restrict__ W3h) {
-    constexpr int G = 4, WPG = CONV_WARPS / G;
+// The pair kernel's BF16 dE/dw takes two terms (it is the sum of two directions).
+template <int H, int AT, int BT>
+__device__ __forceinline__ void chunk_gw_gemm(const ConvDesc& D, const ConvSmem& L, float* smem,
+                                              const __nv_bfloat16* __restrict__ W3h) {
+    constexpr int G = 4, WPG = CONV_WARPS / G, MT = AT > BT ? AT : BT;
     constexpr int NTW = (H / 8) / WPG;         // n tiles per warp (4 or 2)
     static_assert(EC == 16, "one m tile of edges");
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5, g = lane >> 2, tq = lane & 3;
@@ -349,39 +376,50 @@ __device__ __forceinline__ void chunk_gw_gemm_bf16(const ConvDesc& D, const Conv
     float* s_w = smem + L.w;                   // dE/dw, [EC][Wpad]
     float* s_gH = smem + L.gH;                 // [H][EC]
     const int W = D.W, nkb = W / 32;
+    const size_t term = (size_t)W * H;
     const int kb0 = nkb * grp / G, kb1 = nkb * (grp + 1) / G;
     __syncthreads();                           // every warp's dE/dw of phase E is in s_w
     float c[NTW][4];
 #pragma unroll
     for (int j = 0; j < NTW; ++j) c[j][0] = c[j][1] = c[j][2] = c[j][3] = 0.f;
     for (int kb = kb0; kb < kb1; ++kb) {
-        uint4 bv[NTW];
+        uint4 bv[NTW][BT];
 #pragma unroll
         for (int j = 0; j < NTW; ++j)
-            bv[j] = __ldg(reinterpret_cast<const uint4*>(W3h + (size_t)((wq * NTW + j) * 8 + g) * W + kb * 32) + tq);
+#pragma unroll
+            for (int z = 0; z < BT; ++z)
+                bv[j][z] = __ldg(reinterpret_cast<const uint4*>(W3h + z * term + (size_t)((wq * NTW + j) * 8 + g) * W + kb * 32) + tq);
+        float ct[NTW][4] = {}, cs[NTW][4] = {};    // FP32: leading and small products of this block
         // k step ks covers words kb*16 + 4 tq + 2 ks (+1): columns 32 kb + 8 tq + 4 ks .. + 3
 #pragma unroll
         for (int ks = 0; ks < 2; ++ks) {
             const int c0 = kb * 32 + 8 * tq + 4 * ks;
             const float4 r0 = *reinterpret_cast<const float4*>(s_w + g * D.Wpad + c0);
             const float4 r1 = *reinterpret_cast<const float4*>(s_w + (g + 8) * D.Wpad + c0);
-            const uint32_t a[4] = {pack_bf16(r0.x, r0.y), pack_bf16(r1.x, r1.y), pack_bf16(r0.z, r0.w),
-                                   pack_bf16(r1.z, r1.w)};
-            uint32_t al[4];
-            if constexpr (SPLIT) {                 // the remainders x - bf16(x)
-                const float4 h0 = unpack_bf16x4(a[0], a[2]), h1 = unpack_bf16x4(a[1], a[3]);
-                al[0] = pack_bf16(r0.x - h0.x, r0.y - h0.y);
-                al[1] = pack_bf16(r1.x - h1.x, r1.y - h1.y);
-                al[2] = pack_bf16(r0.z - h0.z, r0.w - h0.w);
-                al[3] = pack_bf16(r1.z - h1.z, r1.w - h1.w);
-            }
+            uint32_t a[4][AT];
+            bf16_terms<AT>(r0.x, r0.y, a[0]);
+            bf16_terms<AT>(r1.x, r1.y, a[1]);
+            bf16_terms<AT>(r0.z, r0.w, a[2]);
+            bf16_terms<AT>(r1.z, r1.w, a[3]);
 #pragma unroll
-            for (int j = 0; j < NTW; ++j) {
-                const uint32_t* bw = reinterpret_cast<const uint32_t*>(&bv[j]);
-                const uint32_t b[2] = {bw[2 * ks], bw[2 * ks + 1]};
-                mma_bf16(c[j], a, b);
-                if constexpr (SPLIT) mma_bf16(c[j], al, b);
-            }
+            for (int o = MT - 1; o >= 0; --o)
+#pragma unroll
+                for (int z = 0; z <= o; ++z) {
+                    if (z >= AT || o - z >= BT) continue;
+                    const uint32_t az[4] = {a[0][z < AT ? z : 0], a[1][z < AT ? z : 0], a[2][z < AT ? z : 0], a[3][z < AT ? z : 0]};
+#pragma unroll
+                    for (int j = 0; j < NTW; ++j) {
+                        const uint32_t* bw = reinterpret_cast<const uint32_t*>(&bv[j][o - z < BT ? o - z : 0]);
+                        const uint32_t b[2] = {bw[2 * ks], bw[2 * ks + 1]};
+                        mma_bf16(MT < 3 ? c[j] : (o > 0 ? cs[j] : ct[j]), az, b);
+                    }
+                }
+        }
+        if constexpr (MT == 3) {
+#pragma unroll
+            for (int j = 0; j < NTW; ++j)
+#pragma unroll
+                for (int q = 0; q < 4; ++q) c[j][q] += ct[j][q] + cs[j][q];
         }
     }
     __syncthreads();                           // the partials overwrite s_w
@@ -400,55 +438,60 @@ __device__ __forceinline__ void chunk_gw_gemm_bf16(const ConvDesc& D, const Conv
     __syncthreads();
 }
 
-// Hidden layer of the radial MLP on tensor cores (BF16 path):
-//   out[k_out][e] = sum_k in[k][e] B[k][k_out], B given N-major ([k_out][k]) as a
-//   hi + lo BF16 pair, the input as one BF16 value; two MMAs per k step (in*hi, in*lo).
+// Hidden layer of the radial MLP on tensor cores:
+//   out[k_out][e] = sum_k in[k][e] B[k][k_out], B given N-major ([k_out][k]) in BT
+//   terms, the input in AT terms.
 // The 16 edges of the chunk are one m tile; warps take n tiles of 8 outputs.
-template <int H>
-struct HiddenB {                                   // B fragments of one n tile, hi and lo
-    uint4 hi[H / 32], lo[H / 32];
+template <int H, int BT = 2>
+struct HiddenB {                                   // B fragments of one n tile
+    uint4 b[BT][H / 32];
 };
 
-template <int H>
-__device__ __forceinline__ void hidden_load(const __nv_bfloat16* __restrict__ Bn, int nt, HiddenB<H>& b) {
+template <int H, int BT>
+__device__ __forceinline__ void hidden_load(const __nv_bfloat16* __restrict__ Bn, int nt, HiddenB<H, BT>& b) {
     constexpr int NV = H / 32;
     const int lane = threadIdx.x & 31, g = lane >> 2, tq = lane & 3;
-    const uint4* hi = reinterpret_cast<const uint4*>(Bn + (size_t)(nt * 8 + g) * H) + tq * NV;
-    const uint4* lo = reinterpret_cast<const uint4*>(Bn + (size_t)H * H + (size_t)(nt * 8 + g) * H) + tq * NV;
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        b.hi[v] = __ldg(hi + v);
-        b.lo[v] = __ldg(lo + v);
+    for (int z = 0; z < BT; ++z) {
+        const uint4* p = reinterpret_cast<const uint4*>(Bn + (size_t)z * H * H + (size_t)(nt * 8 + g) * H) + tq * NV;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) b.b[z][v] = __ldg(p + v);
     }
 }
 
-// SPLIT: the input also enters as a hi + lo BF16 pair (in_lo * W2_hi added).
-template <int H, bool SPLIT = false>
-__device__ __forceinline__ void hidden_mma(const float* __restrict__ s_in, const HiddenB<H>& bf, float (&c)[4]) {
-    constexpr int KSN = H / 16;
+template <int H, int AT = 1, int BT = 2>
+__device__ __forceinline__ void hidden_mma(const float* __restrict__ s_in, const HiddenB<H, BT>& bf, float (&c)[4]) {
+    constexpr int KSN = H / 16, MT = AT > BT ? AT : BT;
     const int lane = threadIdx.x & 31, g = lane >> 2, tq = lane & 3;
     c[0] = c[1] = c[2] = c[3] = 0.f;
-    const uint32_t* wh = reinterpret_cast<const uint32_t*>(bf.hi);
-    const uint32_t* wl = reinterpret_cast<const uint32_t*>(bf.lo);
+    float cs[4] = {};
 #pragma unroll
     for (int ks = 0; ks < KSN; ++ks) {
-        const int k0 = 2 * (tq * 2 * KSN + 2 * ks), k1 = k0 + 2;
-        const uint32_t a[4] = {pack_bf16(s_in[hk<H>(k0, g)], s_in[hk<H>(k0 + 1, g)]),
-                               pack_bf16(s_in[hk<H>(k0, g + 8)], s_in[hk<H>(k0 + 1, g + 8)]),
-                               pack_bf16(s_in[hk<H>(k1, g)], s_in[hk<H>(k1 + 1, g)]),
-                               pack_bf16(s_in[hk<H>(k1, g + 8)], s_in[hk<H>(k1 + 1, g + 8)])};
-        const uint32_t b[2] = {wh[2 * ks], wh[2 * ks + 1]};
-        const uint32_t b2[2] = {wl[2 * ks], wl[2 * ks + 1]};
-        mma_bf16(c, a, b);
-        mma_bf16(c, a, b2);
-        if constexpr (SPLIT) {
-            const float4 h0 = unpack_bf16x4(a[0], a[2]), h1 = unpack_bf16x4(a[1], a[3]);
-            const uint32_t al[4] = {pack_bf16(s_in[hk<H>(k0, g)] - h0.x, s_in[hk<H>(k0 + 1, g)] - h0.y),
-                                    pack_bf16(s_in[hk<H>(k0, g + 8)] - h1.x, s_in[hk<H>(k0 + 1, g + 8)] - h1.y),
-                                    pack_bf16(s_in[hk<H>(k1, g)] - h0.z, s_in[hk<H>(k1 + 1, g)] - h0.w),
-                                    pack_bf16(s_in[hk<H>(k1, g + 8)] - h1.z, s_in[hk<H>(k1 + 1, g + 8)] - h1.w)};
-            mma_bf16(c, al, b);
+        float ct[4] = {};
+        uint32_t a[4][AT];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int k = 2 * (tq * 2 * KSN + 2 * ks) + 2 * (q >> 1), e = g + 8 * (q & 1);
+            bf16_terms<AT>(s_in[hk<H>(k, e)], s_in[hk<H>(k + 1, e)], a[q]);
         }
+#pragma unroll
+        for (int o = MT - 1; o >= 0; --o)
+#pragma unroll
+            for (int z = 0; z <= o; ++z) {
+                if (z >= AT || o - z >= BT) continue;
+                const uint32_t* w = reinterpret_cast<const uint32_t*>(bf.b[o - z < BT ? o - z : 0]);
+                const uint32_t az[4] = {a[0][z < AT ? z : 0], a[1][z < AT ? z : 0], a[2][z < AT ? z : 0], a[3][z < AT ? z : 0]};
+                const uint32_t b[2] = {w[2 * ks], w[2 * ks + 1]};
+                mma_bf16(MT < 3 ? c : (o > 0 ? cs : ct), az, b);
+            }
+        if constexpr (MT == 3) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) c[q] += ct[q];
+        }
+    }
+    if constexpr (MT == 3) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) c[q] += cs[q];
     }
 }
 
@@ -481,7 +524,6 @@ __device__ __forceinline__ void load_W1(const ConvDesc& D, const ConvSmem& L, fl
 template <int H, bool BF, int LMAX>
 __device__ __forceinline__ void chunk_prologue(const ConvDesc& D, const ConvSmem& L, float* smem,
                                                int c0, int ne, const EdgePrefetch& pf,
-                                               const float* __restrict__ W2,
                                                const __nv_bfloat16* __restrict__ W2T_h) {
     const int t = threadIdx.x, warp = t >> 5;
     int* s_src = reinterpret_cast<int*>(smem + L.src);
@@ -538,103 +580,19 @@ __device__ __forceinline__ void chunk_prologue(const ConvDesc& D, const ConvSmem
         path_G<LMAX>(D.paths[p].kind, s_Y + e * y_stride<LMAX>(), s_G + e * D.nG + D.paths[p].g_off);
     }
     __syncthreads();
-    if constexpr (BF) {          // A2 = H1 @ W2 on tensor cores, H2 = silu(A2)
-        const int lane = t & 31, g = lane >> 2, tq = lane & 3;
-        if (warp < H / 8) {
-            const int nt = warp;
-            float c[4];
-            HiddenB<H> hb;
-            hidden_load<H>(W2T_h, nt, hb);
-            hidden_mma<H>(s_H1, hb, c);
-            const int j = nt * 8 + 2 * tq;
-            const int o[4] = {hk<H>(j, g), hk<H>(j + 1, g), hk<H>(j, g + 8), hk<H>(j + 1, g + 8)};
+    if (warp < H / 8) {          // A2 = H1 @ W2, H2 = silu(A2)
+        const int lane = t & 31, g = lane >> 2, tq = lane & 3, nt = warp;
+        constexpr int AT = BF ? 1 : 3, BT = BF ? 2 : 3;
+        float c[4];
+        HiddenB<H, BT> hb;
+        hidden_load<H, BT>(W2T_h, nt, hb);
+        hidden_mma<H, AT, BT>(s_H1, hb, c);
+        const int j = nt * 8 + 2 * tq;
+        const int o[4] = {hk<H>(j, g), hk<H>(j + 1, g), hk<H>(j, g + 8), hk<H>(j + 1, g + 8)};
 #pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                s_A2[o[q]] = c[q];
-                s_H2[o[q]] = siluf_(c[q]);
-            }
-        }
-    } else {
-        // A2 = H1 @ W2, H2 = silu(A2): each thread computes 4 hidden units of one edge
-        for (int idx = t; idx < (H / 4) * EC; idx += CONV_THREADS) {
-            const int jq = idx / EC, e = idx % EC;
-            float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f;
-#pragma unroll 8
-            for (int k = 0; k < H; ++k) {
-                const float4 b = __ldg(reinterpret_cast<const float4*>(W2 + k * H) + jq);
-                const float a = s_H1[hk<H>(k, e)];
-                a0 = fmaf(a, b.x, a0);
-                a1 = fmaf(a, b.y, a1);
-                a2 = fmaf(a, b.z, a2);
-                a3 = fmaf(a, b.w, a3);
-            }
-            const float av[4] = {a0, a1, a2, a3};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int o = hk<H>(4 * jq + q, e);
-                s_A2[o] = av[q];
-                s_H2[o] = siluf_(av[q]);
-            }
-        }
-    }
-    __syncthreads();
-}
-
-// Phase D (FP32): w[e][c] = sum_k H2[k][e] W3[k][c] for all W columns.
-template <int H>
-__device__ __forceinline__ void chunk_w_gemm_f32(const ConvDesc& D, const ConvSmem& L, float* smem,
-                                                 const float* __restrict__ W3) {
-    constexpr int NEG = EC / 4;                 // groups of 4 edges
-    constexpr int NCG = CONV_THREADS / NEG;     // column-quad threads per edge group
-    constexpr int NQ = DCOLS / (4 * NCG);       // column quads per thread and pass
-    const int t = threadIdx.x;
-    const int eg = t / NCG, cg = t % NCG;
-    const float* s_H2 = smem + L.H2;
-    float4* st4 = reinterpret_cast<float4*>(smem + L.stage);   // [KS][DCOLS/4]
-    float* s_w = smem + L.w;
-    const int W = D.W;
-    for (int cb = 0; cb < W; cb += DCOLS) {
-        float acc[4][NQ][4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int j = 0; j < NQ; ++j)
-#pragma unroll
-                for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.0f;
-        for (int k0 = 0; k0 < H; k0 += KS) {
-            __syncthreads();
-            for (int i = t; i < KS * (DCOLS / 4); i += CONV_THREADS) {
-                const int kk = i / (DCOLS / 4), q = i % (DCOLS / 4);
-                const int col = cb + 4 * q;
-                float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (col < W) v = __ldg(reinterpret_cast<const float4*>(W3 + (size_t)(k0 + kk) * W + col));
-                st4[i] = v;
-            }
-            __syncthreads();
-#pragma unroll
-            for (int kk = 0; kk < KS; ++kk) {
-                const float4 a = *reinterpret_cast<const float4*>(s_H2 + hk<H>(k0 + kk, 4 * eg));
-                const float av[4] = {a.x, a.y, a.z, a.w};
-#pragma unroll
-                for (int j = 0; j < NQ; ++j) {
-                    const float4 b = st4[kk * (DCOLS / 4) + cg + NCG * j];
-                    const float bv[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i)
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) acc[i][j][q] = fmaf(av[i], bv[q], acc[i][j][q]);
-                }
-            }
-        }
-#pragma unroll
-        for (int j = 0; j < NQ; ++j) {
-            const int col = cb + 4 * (cg + NCG * j);
-            if (col < W) {
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    *reinterpret_cast<float4*>(s_w + (4 * eg + i) * D.Wpad + col) =
-                        make_float4(acc[i][j][0], acc[i][j][1], acc[i][j][2], acc[i][j][3]);
-            }
+        for (int q = 0; q < 4; ++q) {
+            s_A2[o[q]] = c[q];
+            s_H2[o[q]] = siluf_(c[q]);
         }
     }
     __syncthreads();
@@ -679,73 +637,6 @@ __device__ __forceinline__ void load_G(const float* __restrict__ src, float* G) 
         G[4 * i + 3] = v.w;
     }
 }
-
-template <int H>
-__device__ __forceinline__ void chunk_gw_gemm_f32(const ConvDesc& D, const ConvSmem& L, float* smem,
-                                                  const float* __restrict__ W3T) {
-    constexpr int KQ = H / 4;                 // k quads
-    constexpr int EGN = 128 / KQ;             // edge groups per half
-    constexpr int EPT = EC / EGN;             // edges per thread
-    const int t = threadIdx.x;
-    const int half = t >> 7, tp = t & 127;
-    const int kq = tp % KQ, eg = tp / KQ;
-    const float* s_w = smem + L.w;
-    float* stage = smem + L.stage;            // [2][CS][H]
-    float acc[EPT][4];
-#pragma unroll
-    for (int i = 0; i < EPT; ++i)
-#pragma unroll
-        for (int q = 0; q < 4; ++q) acc[i][q] = 0.0f;
-    const int W = D.W;
-    for (int cb = 0; cb < W; cb += 2 * CS) {
-        __syncthreads();
-        for (int i = t; i < 2 * CS * (H / 4); i += CONV_THREADS) {
-            const int hh = i / (CS * (H / 4));
-            const int r = i % (CS * (H / 4));
-            const int cc = r / (H / 4), k4 = r % (H / 4);
-            const int c = cb + hh * CS + cc;
-            float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (c < W) v = __ldg(reinterpret_cast<const float4*>(W3T + (size_t)c * H) + k4);
-            reinterpret_cast<float4*>(stage)[i] = v;
-        }
-        __syncthreads();
-        const int cbase = cb + half * CS;
-        const int cn = min(CS, W - cbase);
-        const float* sh = stage + half * CS * H;
-        for (int cc = 0; cc < cn; ++cc) {
-            const float4 b = *reinterpret_cast<const float4*>(sh + cc * H + 4 * kq);
-#pragma unroll
-            for (int i = 0; i < EPT; ++i) {
-                const float a = s_w[(eg * EPT + i) * D.Wpad + cbase + cc];
-                acc[i][0] = fmaf(a, b.x, acc[i][0]);
-                acc[i][1] = fmaf(a, b.y, acc[i][1]);
-                acc[i][2] = fmaf(a, b.z, acc[i][2]);
-                acc[i][3] = fmaf(a, b.w, acc[i][3]);
-            }
-        }
-    }
-    __syncthreads();
-    float* red = stage;                       // [EC][H]
-    if (half == 1) {
-#pragma unroll
-        for (int i = 0; i < EPT; ++i)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) red[(eg * EPT + i) * H + 4 * kq + q] = acc[i][q];
-    }
-    __syncthreads();
-    float* s_gH = smem + L.gH;                // [H][EC]
-    if (half == 0) {
-#pragma unroll
-        for (int i = 0; i < EPT; ++i)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                const int e = eg * EPT + i, k = 4 * kq + q;
-                s_gH[hk<H>(k, e)] = acc[i][q] + red[e * H + k];
-            }
-    }
-    __syncthreads();
-}
-
 
 static inline size_t smem_bytes(const ConvDesc& D, int H, bool bwd, bool bf) {
     return (size_t)conv_smem_layout(D.Wpad, D.WpadB, H, D.nG, D.ys, bwd, bf).total * sizeof(float);

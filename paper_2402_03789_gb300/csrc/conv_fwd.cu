@@ -178,8 +178,7 @@ __device__ __forceinline__ void tp_fwd_chunk(const ConvDesc& D, int ne, const WT
 
 template <int H, bool BF, int LMAX>
 __global__ void __launch_bounds__(CONV_THREADS, conv_ctas_per_sm(LMAX))
-conv_fwd_kernel(const ConvDesc D, const float* __restrict__ W1, const float* __restrict__ W2,
-                const float* __restrict__ W3, const __nv_bfloat16* __restrict__ W3T_h,
+conv_fwd_kernel(const ConvDesc D, const float* __restrict__ W1, const __nv_bfloat16* __restrict__ W3T_h,
                 const __nv_bfloat16* __restrict__ W2T_h, int n_atoms, int n_edges,
                 const int* __restrict__ row_ptr, const int* __restrict__ dst,
                 const int* __restrict__ src, const float4* __restrict__ geom,
@@ -209,10 +208,9 @@ conv_fwd_kernel(const ConvDesc D, const float* __restrict__ W1, const float* __r
     for (int c0 = E0; c0 < E1; c0 += EC) {
         const int ne = min(EC, E1 - c0);
         __syncthreads();
-        chunk_prologue<H, BF, LMAX>(D, L, smem, c0, ne, pf, W2, W2T_h);
+        chunk_prologue<H, BF, LMAX>(D, L, smem, c0, ne, pf, W2T_h);
         pf.fetch(c0 + EC, E1, dst, src, geom, row_ptr);   // next chunk's edges, in flight meanwhile
-        if constexpr (BF) chunk_w_gemm_bf16<H, true>(D, L, smem, W3T_h);
-        else chunk_w_gemm_f32<H>(D, L, smem, W3);
+        chunk_w_gemm<H, BF ? 1 : 3, BF>(D, L, smem, W3T_h);
         switch (D.kind) {
             case 0: tp_fwd_chunk<H, LMAX, 0, WT>(D, ne, s_w, smem + L.G, s_src, s_dst, s_first, x, m); break;
             case 1: tp_fwd_chunk<H, LMAX, 1, WT>(D, ne, s_w, smem + L.G, s_src, s_dst, s_first, x, m); break;
@@ -281,7 +279,7 @@ void launch_conv_fwd(const LayerDev& L, int H, sevennet_precision prec, int64_t 
     const int grid = conv_grid(n_atoms, conv_ctas_per_sm(lm));
     const size_t sm = smem_bytes(L.conv, H, false, prec == SEVENNET_BF16);
 #define SN_LF(HH, BB, LL) conv_fwd_kernel<HH, BB, LL><<<grid, CONV_THREADS, sm, st>>>(             \
-        L.conv, L.mlp0, L.mlp1, L.mlp2, L.mlp2h, L.mlp1Th, (int)n_atoms, (int)n_edges, row_ptr, dst, src, geom, x, m)
+        L.conv, L.mlp0, L.mlp2h, L.mlp1Th, (int)n_atoms, (int)n_edges, row_ptr, dst, src, geom, x, m)
     if (H == 64) {
         if (bf) { if (lm == 3) SN_LF(64, true, 3); else if (lm == 2) SN_LF(64, true, 2); else SN_LF(64, true, 1); }
         else    { if (lm == 3) SN_LF(64, false, 3); else if (lm == 2) SN_LF(64, false, 2); else SN_LF(64, false, 1); }

@@ -694,7 +694,6 @@ sevennet_status st_plan_build(sevennet_model* M, LayerDev& L) {
         L.st[0].t[t].w3 = L.st[1].t[t].w3 = p;
     }
     SN_CUDA(cudaGetLastError());
-    SN_CUDA(cudaStreamSynchronize(nullptr));
     return SEVENNET_OK;
 }
 

@@ -356,16 +356,14 @@ struct LayerDev {
     bool last;
     // device weights, pre-scaled by 1/sqrt(fan_in) (and 1/avg_num_neigh for mlp2)
     float* mlp0 = nullptr;   // [NB][H]
-    float* mlp1 = nullptr;   // [H][H]
-    float* mlp2 = nullptr;   // [H][W]
-    float* mlp0T = nullptr;  // [H][NB]
-    float* mlp1T = nullptr;  // [H][H]
+    float* mlp1T = nullptr;  // [H][H] W2^T
     float* mlp2T = nullptr;  // [W][H]
     uint2* mlp1F = nullptr;  // W2 as B fragments, three BF16 terms (radial.cu)
-    __nv_bfloat16* mlp1h = nullptr;   // [2][H][H] W2 as stored, hi then lo (B operand of gA2 @ W2^T)
-    __nv_bfloat16* mlp1Th = nullptr;  // [2][H][H] W2^T, hi then lo (B operand of H1 @ W2)
-    __nv_bfloat16* mlp2h = nullptr;   // [W][H]  (N-major for mma B operand)
-    __nv_bfloat16* mlp2Th = nullptr;  // [H][W]
+    // three BF16 terms each (the BF16 path reads the first, of W2 the first two)
+    __nv_bfloat16* mlp1h = nullptr;   // [3][H][H] W2 as stored (B operand of gA2 @ W2^T)
+    __nv_bfloat16* mlp1Th = nullptr;  // [3][H][H] W2^T (B operand of H1 @ W2)
+    __nv_bfloat16* mlp2h = nullptr;   // [3][W][H] W3^T (N-major for the mma B operand)
+    __nv_bfloat16* mlp2Th = nullptr;  // [3][H][W] W3
     float* lin1[NL] = {};  float* lin1T[NL] = {};  __nv_bfloat16* lin1h[NL] = {};  __nv_bfloat16* lin1Th[NL] = {};
     float* sc[NL] = {};    float* scT[NL] = {};    __nv_bfloat16* sch[NL] = {};    __nv_bfloat16* scTh[NL] = {};
     float* lin2[NL] = {};  float* lin2T[NL] = {};  __nv_bfloat16* lin2h[NL] = {};  __nv_bfloat16* lin2Th[NL] = {};

@@ -119,19 +119,34 @@ radial_kernel(const ConvDesc D, int64_t cap, const int* __restrict__ count, cons
                 }
             }
         float c[8][4] = {};
-        // (A term, B term), smallest product first; the n tiles are independent chains
-        constexpr int NPR = BF ? 3 : 6;
-        constexpr int pa[6] = {BF ? 1 : 0, BF ? 0 : 2, BF ? 0 : 1, 0, 1, 0}, pb[6] = {BF ? 0 : 2, BF ? 1 : 0, BF ? 0 : 1, 1, 0, 0};
+        // products of terms i + j = o < SPL; the n tiles are independent chains.  FP32: the
+        // leading products of a k step are added by FADD (see conv_common.cuh)
 #pragma unroll
-        for (int q = 0; q < NPR; ++q)
+        for (int o = SPL - 1; o > 0; --o)
 #pragma unroll
-            for (int ks = 0; ks < 4; ++ks)
+            for (int z = 0; z <= o; ++z)
 #pragma unroll
-                for (int nt = 0; nt < 8; ++nt) {
-                    const uint2 b = s_b[pb[q]][nt][ks][lane];
-                    const uint32_t bb[2] = {b.x, b.y};
-                    mma_bf16(c[nt], a[pa[q]][ks], bb);
-                }
+                for (int ks = 0; ks < 4; ++ks)
+#pragma unroll
+                    for (int nt = 0; nt < 8; ++nt) {
+                        const uint2 b = s_b[o - z][nt][ks][lane];
+                        const uint32_t bb[2] = {b.x, b.y};
+                        mma_bf16(c[nt], a[z][ks], bb);
+                    }
+#pragma unroll
+        for (int nt = 0; nt < 8; ++nt) {
+            float t[4][4] = {};
+#pragma unroll
+            for (int ks = 0; ks < 4; ++ks) {
+                const uint2 b = s_b[0][nt][ks][lane];
+                const uint32_t bb[2] = {b.x, b.y};
+                mma_bf16(BF ? c[nt] : t[ks], a[0][ks], bb);
+            }
+            if constexpr (!BF) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) c[nt][q] += (t[0][q] + t[1][q]) + (t[2][q] + t[3][q]);
+            }
+        }
         float o[2][16];                                  // pairs g, g + 8: outputs tq * 16 + [0, 16)
 #pragma unroll
         for (int nt = 0; nt < 8; ++nt)

@@ -689,8 +689,10 @@ sevennet_status model_layer_backward_rest(sevennet_model* M, Workspace* ws, int 
     GemmBatch g{};
     for (int l = 0; l < NL; ++l) {
         if (!L.y_mul[l] || !L.msg_mul[l]) continue;
-        g.p[g.n++] = GemmProb{ws->gy, L.lin2T[l], L.lin2Th[l], ws->m, N, 2 * l + 1, L.y_mul[l], L.msg_mul[l],
-                              L.y_dim, L.y_off[l], L.m_dim, L.msg_off[l], 0};
+        GemmProb p{ws->gy, L.lin2T[l], L.lin2Th[l], ws->m, N, 2 * l + 1, L.y_mul[l], L.msg_mul[l],
+                   L.y_dim, L.y_off[l], L.m_dim, L.msg_off[l], 0};
+        if (pairs) p.c_blk = L.g_blk[l];         // the pair adjoint reads blocked rows
+        g.p[g.n++] = p;
     }
     run_gemm(M, g, prec, st);
     prof_begin(&M->prof, PF_CONV_BWD, st, &ev);
@@ -925,6 +927,26 @@ sevennet_status sevennet_create_model(const sevennet_model_config* cfg, const do
             D.mul_in[l] = L.in_mul[l];
             D.x_off[l] = L.in_off[l];
             if (L.in_mul[l]) D.l1max = l;
+        }
+        // blocked rows of dE/dm: per l1 and 32 channels the values (path, m3) of that block,
+        // 32 channels each, so that a warp's loads are one address plus constants
+        {
+            std::vector<int> blk[NL];
+            int o = 0;
+            for (int l = 0; l < NL; ++l) {
+                D.gb_off[l] = o;
+                int ng = 0;
+                for (int p = D.pbeg[l]; p < D.pend[l]; ++p) ng += 2 * D.paths[p].l3 + 1;
+                int before = 0;
+                for (int p = D.pbeg[l]; p < D.pend[l]; ++p) {
+                    const int l3 = D.paths[p].l3;
+                    for (int g = 0; g < L.in_mul[l] / 32; ++g) blk[l3].push_back(o + g * ng * 32 + before * 32);
+                    before += 2 * l3 + 1;
+                }
+                o += L.in_mul[l] * ng;
+            }
+            for (int l = 0; l < NL; ++l)
+                if (sevennet_status s = dev_upload(M, blk[l], &L.g_blk[l])) return fail(s);
         }
         D.kind = (t == 0 ? 1 : 0) | (L.last ? 2 : 0);
         for (int l1 = 0; l1 <= MAX_LMAX; ++l1) {          // the kernels rely on this order

@@ -9,42 +9,6 @@
 namespace sn {
 
 // ------------------------------------------------------------- adjoint
-// One path of one edge for CPL channels per lane (channels u0 + 32 k): the
-// G matrix and the address arithmetic serve all of them.
-template <int L1, int L2, int L3, int CPL>
-__device__ __forceinline__ void tp_bwd_path(const PathDesc& P, int u0, int e, int v, const float (*xv)[2 * L1 + 1],
-                                            float (*gx)[2 * L1 + 1], float* gY, float* s_w, int Wpad,
-                                            const float* s_G, int nG,
-                                            const float* __restrict__ gm, int m_dim) {
-    constexpr int N1 = 2 * L1 + 1, N3 = 2 * L3 + 1;
-    float* wr = s_w + e * Wpad + P.col0 + u0;
-    const float* gmr = gm + (size_t)v * m_dim + P.m_off + P.m_ch0 + u0;
-    float g[CPL][N3];
-#pragma unroll
-    for (int k = 0; k < CPL; ++k)
-#pragma unroll
-        for (int c = 0; c < N3; ++c) g[k][c] = __ldg(gmr + c * P.m_mul + 32 * k);
-    float G[((N1 * N3 + 3) / 4) * 4];
-    load_G<N1 * N3>(s_G + e * nG + P.g_off, G);
-#pragma unroll
-    for (int k = 0; k < CPL; ++k) {
-        const float wv = wr[32 * k];
-        float gw = 0.0f;
-        float wx[N1];
-#pragma unroll
-        for (int a = 0; a < N1; ++a) {
-            float tt = 0.0f;
-#pragma unroll
-            for (int c = 0; c < N3; ++c) tt = fmaf(G[a * N3 + c], g[k][c], tt);
-            gw = fmaf(xv[k][a], tt, gw);
-            gx[k][a] = fmaf(wv, tt, gx[k][a]);
-            wx[a] = wv * xv[k][a];
-        }
-        wr[32 * k] = gw;             // dE/dw replaces w (same thread, same slot)
-        CG<L1, L2, L3>::gY(wx, g[k], gY + L2 * L2);
-    }
-}
-
 // Fixed-point add of one dE/dx contribution (order-independent sums); the
 // conversion after the kernel reports a sum that received the sentinel.
 __device__ __forceinline__ void gx_fixed_add(unsigned long long* p, float v) {
@@ -52,235 +16,175 @@ __device__ __forceinline__ void gx_fixed_add(unsigned long long* p, float v) {
     atomicAdd(p, (unsigned long long)q);
 }
 
-// All paths of one input irrep l1 for one edge, CPL channels per lane: the
-// channel loads, the path descriptors and the CG code resolve at compile time.
-template <int L1, int LMAX, int KIND, int CPL>
-__device__ __forceinline__ void tp_bwd_block(const ConvDesc& D, int u0, int e, int v, int sidx, float* gY,
-                                             float* s_w, const float* s_G, const float* __restrict__ x,
-                                             const float* __restrict__ gm, unsigned long long* __restrict__ gxo) {
-    using BP = BlockPaths<L1, LMAX, KIND>;
-    constexpr int N1 = 2 * L1 + 1;
-    const int mul = D.mul_in[L1];
-    const float* xr = x + (size_t)sidx * D.x_dim + D.x_off[L1] + u0;
-    unsigned long long* gxr = gxo ? gxo + (size_t)sidx * D.x_dim + D.x_off[L1] + u0 : nullptr;
-    float xv[CPL][N1], gx[CPL][N1];
+// ------------------------------------------------------------- tensor product
+// Units are edges (DIRS = 1) or unordered pairs (DIRS = 2).  An edge e (receiver v,
+// sender w, d = r_w + S cell - r_v) and its reverse (receiver w, sender v, -d) share
+// the radial weights w_e, which depend on |d| only, and Y_l(-d/r) = (-1)^l Y_l(d/r),
+// so G of the reverse is (-1)^l2 G.  The pair kernel runs the radial MLP, the G
+// matrices and their adjoints once per pair and the tensor product once per
+// direction: direction 0 is e itself, direction 1 takes dE/dm of w times (-1)^l2 and
+// x of v, which gives the reverse edge's products expressed through Y(d/r).  dE/dw,
+// and dE/dY w.r.t. Y(d/r), are the sums over both directions.
+//
+// One path, a channel per lane:
+//   t[m1] = sum_{m3} G[m1][m3] g[m3],  dE/dw += x[m1] t[m1],  dE/dx[m1] += w t[m1],
+//   S[m1][m3] += w x[m1] g[m3] over both directions, and dE/dY += C : S once
+// (the coupling applied per direction cost two instructions a coefficient, half of
+// the phase's arithmetic).  Y of degree 0 is constant: no S for l2 = 0.
+template <int L1, int L2, int L3, int DIRS, int NCH, int OFF, int NG>
+__device__ __forceinline__ void tp_bwd_path(const PathDesc& P, int u0, int e, const float (&x)[DIRS * NCH][2 * L1 + 1],
+                                            float (&gx)[DIRS * NCH][2 * L1 + 1], const float (&g)[DIRS * NCH][NG],
+                                            float* gY, float* s_w, int Wpad, const float* s_G, int nG) {
+    constexpr int N1 = 2 * L1 + 1, N3 = 2 * L3 + 1;
+    float* wr = s_w + e * Wpad + P.col0 + u0;
+    float wv[NCH], gw[NCH];
 #pragma unroll
-    for (int k = 0; k < CPL; ++k)
-#pragma unroll
-        for (int a = 0; a < N1; ++a) {
-            xv[k][a] = __ldg(xr + a * mul + 32 * k);
-            gx[k][a] = 0.0f;
-        }
-    static_for<BP::list.n>([&](auto I) {
-        constexpr int i = decltype(I)::value;
-        tp_bwd_path<L1, BP::list.l2[i], BP::list.l3[i], CPL>(D.paths[BP::begin + i], u0, e, v, xv, gx, gY,
-                                                             s_w, D.Wpad, s_G, D.nG, gm, D.m_dim);
-    });
-    if (gxr) {                                   // null: the block's dE/dx is not needed
-#pragma unroll
-        for (int k = 0; k < CPL; ++k)
-#pragma unroll
-            for (int a = 0; a < N1; ++a) gx_fixed_add(gxr + a * mul + 32 * k, gx[k][a]);
+    for (int h = 0; h < NCH; ++h) {
+        wv[h] = wr[32 * h];
+        gw[h] = 0.0f;
     }
-}
-
-template <int L1, int LMAX, int KIND, int MAXC>
-__device__ __forceinline__ void tp_bwd_l1(const ConvDesc& D, int lane, int e, int v, int sidx,
-                                          float* gY, float* s_w, const float* s_G,
-                                          const float* __restrict__ x,
-                                          const float* __restrict__ gm, unsigned long long* __restrict__ gxo) {
-    if constexpr (BlockPaths<L1, LMAX, KIND>::list.n > 0) {
-        const int mul = D.mul_in[L1];
-        for (int ub = 0; ub < mul;) {
-            const int left = (mul - ub) / 32;
-            if (MAXC >= 4 && left >= 4) {
-                tp_bwd_block<L1, LMAX, KIND, (MAXC >= 4 ? 4 : 1)>(D, ub + lane, e, v, sidx, gY, s_w, s_G, x, gm, gxo);
-                ub += 128;
-            } else if (MAXC >= 2 && left >= 2) {
-                tp_bwd_block<L1, LMAX, KIND, (MAXC >= 2 ? 2 : 1)>(D, ub + lane, e, v, sidx, gY, s_w, s_G, x, gm, gxo);
-                ub += 64;
-            } else {
-                tp_bwd_block<L1, LMAX, KIND, 1>(D, ub + lane, e, v, sidx, gY, s_w, s_G, x, gm, gxo);
-                ub += 32;
+    float G[((N1 * N3 + 3) / 4) * 4];
+    load_G<N1 * N3>(s_G + e * nG + P.g_off, G);
+    float S[N1 * N3];
+#pragma unroll
+    for (int a = 0; a < N1; ++a)
+#pragma unroll
+        for (int k = 0; k < DIRS * NCH; ++k) {
+            const int h = k % NCH;
+            const bool neg = k >= NCH && (L2 & 1);       // G of the reverse edge
+            float t = 0.0f;
+#pragma unroll
+            for (int c = 0; c < N3; ++c) t = fmaf(G[a * N3 + c], g[k][OFF + c], t);
+            if (neg) t = -t;
+            gw[h] = fmaf(x[k][a], t, gw[h]);
+            gx[k][a] = fmaf(wv[h], t, gx[k][a]);
+            if constexpr (L2 > 0) {
+                const float wx = (neg ? -wv[h] : wv[h]) * x[k][a];
+#pragma unroll
+                for (int c = 0; c < N3; ++c)
+                    S[a * N3 + c] = k == 0 ? wx * g[0][OFF + c] : fmaf(wx, g[k][OFF + c], S[a * N3 + c]);
             }
         }
+    if constexpr (L2 > 0) CG<L1, L2, L3>::S(S, gY + L2 * L2);
+#pragma unroll
+    for (int h = 0; h < NCH; ++h) wr[32 * h] = gw[h];    // dE/dw of the unit replaces w (same thread, same slot)
+}
+
+template <int L1, int LMAX, int KIND>
+__host__ __device__ constexpr int tp_g_off(int i) {        // dE/dm values of the paths before path i
+    const PathList p = path_list(L1, LMAX, KIND);
+    int o = 0;
+    for (int k = 0; k < i; ++k) o += 2 * p.l3[k] + 1;
+    return o;
+}
+
+// All paths of one input irrep l1 over 32 channels of one unit: the channel loads,
+// the path descriptors and the CG code resolve at compile time.  Every dE/dm value
+// of the block is loaded before the first path.  The pair kernel reads blocked rows
+// of dE/dm ([l1][32 channels][path, m3][channel], written by the linear_2 adjoint):
+// in the message layout the address arithmetic of its loads was a fifth of the
+// kernel's instructions.  24,000 atoms BF16, adjoints of 5 layers: 12.84 ms with a
+// load wave per path and C applied per direction, 13.18 ms with S and loads up front
+// in the message layout, 12.25 ms with blocked rows.  The per-edge kernel gets dE/dm
+// from its caller, in the message layout.  Scalars (at most 3 x 2 registers a path)
+// run two channels a lane where 64 are left, which halves their reads of G.
+template <int L1, int LMAX, int KIND, int DIRS, int NCH>
+__device__ __forceinline__ void tp_bwd_block(const ConvDesc& D, int u0, int e, const int (&recv)[DIRS],
+                                             const int (&send)[DIRS], float* gY, float* s_w, const float* s_G,
+                                             const float* __restrict__ x, const float* __restrict__ gm,
+                                             unsigned long long* __restrict__ gxo) {
+    using BP = BlockPaths<L1, LMAX, KIND>;
+    constexpr int N1 = 2 * L1 + 1, NG = tp_g_off<L1, LMAX, KIND>(BP::list.n), K = DIRS * NCH;
+    const int mul = D.mul_in[L1];
+    float xv[K][N1], gx[K][N1], g[K][NG];
+#pragma unroll
+    for (int q = 0; q < DIRS; ++q) {
+        if constexpr (DIRS == 2) {               // blocked rows
+            const int lane = threadIdx.x & 31;
+            const float* gr = gm + (size_t)recv[q] * D.m_dim + D.gb_off[L1] + (u0 - lane) * NG + lane;
+#pragma unroll
+            for (int h = 0; h < NCH; ++h)
+#pragma unroll
+                for (int j = 0; j < NG; ++j) g[q * NCH + h][j] = __ldg(gr + 32 * (h * NG + j));
+        } else {
+            const float* gr = gm + (size_t)recv[q] * D.m_dim + u0;
+            static_for<BP::list.n>([&](auto I) {
+                constexpr int i = decltype(I)::value, o = tp_g_off<L1, LMAX, KIND>(i), N3 = 2 * BP::list.l3[i] + 1;
+                const PathDesc& P = D.paths[BP::begin + i];
+#pragma unroll
+                for (int c = 0; c < N3; ++c)
+#pragma unroll
+                    for (int h = 0; h < NCH; ++h)
+                        g[q * NCH + h][o + c] = __ldg(gr + P.m_off + P.m_ch0 + c * P.m_mul + 32 * h);
+            });
+        }
+        const float* xr = x + (size_t)send[q] * D.x_dim + D.x_off[L1] + u0;
+#pragma unroll
+        for (int a = 0; a < N1; ++a)
+#pragma unroll
+            for (int h = 0; h < NCH; ++h) {
+                xv[q * NCH + h][a] = __ldg(xr + a * mul + 32 * h);
+                gx[q * NCH + h][a] = 0.0f;
+            }
+    }
+    static_for<BP::list.n>([&](auto I) {
+        constexpr int i = decltype(I)::value;
+        tp_bwd_path<L1, BP::list.l2[i], BP::list.l3[i], DIRS, NCH, tp_g_off<L1, LMAX, KIND>(i), NG>(
+            D.paths[BP::begin + i], u0, e, xv, gx, g, gY, s_w, D.Wpad, s_G, D.nG);
+    });
+    if (gxo) {                                   // null: the block's dE/dx is not needed
+#pragma unroll
+        for (int q = 0; q < DIRS; ++q) {
+            unsigned long long* o = gxo + (size_t)send[q] * D.x_dim + D.x_off[L1] + u0;
+#pragma unroll
+            for (int a = 0; a < N1; ++a)
+#pragma unroll
+                for (int h = 0; h < NCH; ++h) gx_fixed_add(o + a * mul + 32 * h, gx[q * NCH + h][a]);
+        }
     }
 }
 
-// Phase E of the adjoint for every edge of the chunk (warp per edge).
-template <int LMAX, int KIND, int MAXC>
+// Phase E for every unit of the chunk, a warp per unit (slot e: receiver s_dst[e],
+// sender s_src[e]).
+template <int LMAX, int KIND, int DIRS>
 __device__ __forceinline__ void tp_bwd_chunk(const ConvDesc& D, int ne, const int* s_dst, const int* s_src,
                                              float* s_w, const float* s_G, float* s_gY,
                                              const float* __restrict__ x, const float* __restrict__ gm,
                                              unsigned long long* __restrict__ gx) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int e = warp; e < ne; e += CONV_WARPS) {
-        const int v = s_dst[e], sidx = s_src[e];
+        int recv[DIRS], send[DIRS];
+        recv[0] = s_dst[e];
+        send[0] = s_src[e];
+        if constexpr (DIRS == 2) {
+            recv[1] = send[0];
+            send[1] = recv[0];
+        }
         constexpr int NYS = LMAX >= 3 ? 16 : 9;
         float gY[NYS];
 #pragma unroll
         for (int i = 0; i < NYS; ++i) gY[i] = 0.0f;
-        tp_bwd_l1<0, LMAX, KIND, MAXC>(D, lane, e, v, sidx, gY, s_w, s_G, x, gm, gx);
-        tp_bwd_l1<1, LMAX, KIND, MAXC>(D, lane, e, v, sidx, gY, s_w, s_G, x, gm, gx);
-        if constexpr (LMAX >= 2) tp_bwd_l1<2, LMAX, KIND, MAXC>(D, lane, e, v, sidx, gY, s_w, s_G, x, gm, gx);
-        if constexpr (LMAX >= 3) tp_bwd_l1<3, LMAX, KIND, MAXC>(D, lane, e, v, sidx, gY, s_w, s_G, x, gm, gx);
+        static_for<LMAX + 1>([&](auto Lc) {
+            constexpr int L1 = decltype(Lc)::value;
+            if constexpr (BlockPaths<L1, LMAX, KIND>::list.n > 0) {
+                int ub = 0;
+                if constexpr (L1 == 0 && LMAX <= 2) {    // short paths: two channels a lane
+#pragma unroll 1
+                    for (; ub + 64 <= D.mul_in[L1]; ub += 64)
+                        tp_bwd_block<L1, LMAX, KIND, DIRS, 2>(D, ub + lane, e, recv, send, gY, s_w, s_G, x, gm, gx);
+                }
+#pragma unroll 1
+                for (; ub < D.mul_in[L1]; ub += 32)
+                    tp_bwd_block<L1, LMAX, KIND, DIRS, 1>(D, ub + lane, e, recv, send, gY, s_w, s_G, x, gm, gx);
+            }
+        });
         constexpr int NY = (LMAX + 1) * (LMAX + 1);
 #pragma unroll
-        for (int i = 0; i < NY; ++i) gY[i] = warp_sum(gY[i]);
+        for (int i = 1; i < NY; ++i) gY[i] = warp_sum(gY[i]);
         if (lane < NYS) {
             float val = 0.0f;
 #pragma unroll
-            for (int i = 0; i < NY; ++i) if (lane == i) val = gY[i];
-            s_gY[e * y_stride<LMAX>() + lane] = val;
-        }
-    }
-}
-
-// ------------------------------------------------------------- unordered pairs
-// An edge e (receiver v, sender w, d = r_w + S cell - r_v) and its reverse
-// (receiver w, sender v, -d) share the radial weights w_e, which depend on |d|
-// only, and Y_l(-d/r) = (-1)^l Y_l(d/r), so G of the reverse is (-1)^l2 G.  The
-// pair kernel runs the radial MLP, the G matrices and their adjoints once per
-// pair and the tensor product once per direction: direction a is e itself,
-// direction b takes dE/dm of w times (-1)^l2 and x of v, which gives the
-// reverse edge's products expressed through Y(d/r).  dE/dw, and dE/dY w.r.t.
-// Y(d/r), are the sums over both directions.
-template <int L1, int L2, int L3, int CPL>
-__device__ __forceinline__ void tp_bwd_path_pair(const PathDesc& P, int u0, int e, int v, int w,
-                                                 const float (*xa)[2 * L1 + 1], const float (*xb)[2 * L1 + 1],
-                                                 float (*gxa)[2 * L1 + 1], float (*gxb)[2 * L1 + 1], float* gY,
-                                                 float* s_w, int Wpad, const float* s_G, int nG,
-                                                 const float* __restrict__ gm, int m_dim) {
-    constexpr int N1 = 2 * L1 + 1, N3 = 2 * L3 + 1;
-    constexpr float sb = (L2 & 1) ? -1.0f : 1.0f;
-    float* wr = s_w + e * Wpad + P.col0 + u0;
-    const float* gma = gm + (size_t)v * m_dim + P.m_off + P.m_ch0 + u0;
-    const float* gmb = gm + (size_t)w * m_dim + P.m_off + P.m_ch0 + u0;
-    float ga[CPL][N3], gb[CPL][N3];
-#pragma unroll
-    for (int k = 0; k < CPL; ++k)
-#pragma unroll
-        for (int c = 0; c < N3; ++c) {
-            ga[k][c] = __ldg(gma + c * P.m_mul + 32 * k);
-            gb[k][c] = sb * __ldg(gmb + c * P.m_mul + 32 * k);
-        }
-    float G[((N1 * N3 + 3) / 4) * 4];
-    load_G<N1 * N3>(s_G + e * nG + P.g_off, G);
-#pragma unroll
-    for (int k = 0; k < CPL; ++k) {
-        const float wv = wr[32 * k];
-        float gw = 0.0f;
-        float wx[N1];
-#pragma unroll
-        for (int a = 0; a < N1; ++a) {
-            float tt = 0.0f;
-#pragma unroll
-            for (int c = 0; c < N3; ++c) tt = fmaf(G[a * N3 + c], ga[k][c], tt);
-            gw = fmaf(xa[k][a], tt, gw);
-            gxa[k][a] = fmaf(wv, tt, gxa[k][a]);
-            wx[a] = wv * xa[k][a];
-        }
-        CG<L1, L2, L3>::gY(wx, ga[k], gY + L2 * L2);
-#pragma unroll
-        for (int a = 0; a < N1; ++a) {
-            float tt = 0.0f;
-#pragma unroll
-            for (int c = 0; c < N3; ++c) tt = fmaf(G[a * N3 + c], gb[k][c], tt);
-            gw = fmaf(xb[k][a], tt, gw);
-            gxb[k][a] = fmaf(wv, tt, gxb[k][a]);
-            wx[a] = wv * xb[k][a];
-        }
-        CG<L1, L2, L3>::gY(wx, gb[k], gY + L2 * L2);
-        wr[32 * k] = gw;             // dE/dw of the pair replaces w
-    }
-}
-
-template <int L1, int LMAX, int KIND, int CPL>
-__device__ __forceinline__ void tp_bwd_block_pair(const ConvDesc& D, int u0, int e, int v, int w, float* gY,
-                                                  float* s_w, const float* s_G, const float* __restrict__ x,
-                                                  const float* __restrict__ gm,
-                                                  unsigned long long* __restrict__ gxo) {
-    using BP = BlockPaths<L1, LMAX, KIND>;
-    constexpr int N1 = 2 * L1 + 1;
-    const int mul = D.mul_in[L1];
-    const float* xra = x + (size_t)w * D.x_dim + D.x_off[L1] + u0;     // direction a: sender w
-    const float* xrb = x + (size_t)v * D.x_dim + D.x_off[L1] + u0;     // direction b: sender v
-    float xa[CPL][N1], xb[CPL][N1], gxa[CPL][N1], gxb[CPL][N1];
-#pragma unroll
-    for (int k = 0; k < CPL; ++k)
-#pragma unroll
-        for (int a = 0; a < N1; ++a) {
-            xa[k][a] = __ldg(xra + a * mul + 32 * k);
-            xb[k][a] = __ldg(xrb + a * mul + 32 * k);
-            gxa[k][a] = 0.0f;
-            gxb[k][a] = 0.0f;
-        }
-    static_for<BP::list.n>([&](auto I) {
-        constexpr int i = decltype(I)::value;
-        tp_bwd_path_pair<L1, BP::list.l2[i], BP::list.l3[i], CPL>(D.paths[BP::begin + i], u0, e, v, w, xa, xb,
-                                                                  gxa, gxb, gY, s_w, D.Wpad, s_G, D.nG, gm,
-                                                                  D.m_dim);
-    });
-    if (gxo) {                                   // null: the block's dE/dx is not needed
-        unsigned long long* ra = gxo + (size_t)w * D.x_dim + D.x_off[L1] + u0;
-        unsigned long long* rb = gxo + (size_t)v * D.x_dim + D.x_off[L1] + u0;
-#pragma unroll
-        for (int k = 0; k < CPL; ++k)
-#pragma unroll
-            for (int a = 0; a < N1; ++a) {
-                gx_fixed_add(ra + a * mul + 32 * k, gxa[k][a]);
-                gx_fixed_add(rb + a * mul + 32 * k, gxb[k][a]);
-            }
-    }
-}
-
-template <int L1, int LMAX, int KIND, int MAXC>
-__device__ __forceinline__ void tp_bwd_l1_pair(const ConvDesc& D, int lane, int e, int v, int w, float* gY,
-                                               float* s_w, const float* s_G, const float* __restrict__ x,
-                                               const float* __restrict__ gm, unsigned long long* __restrict__ gxo) {
-    if constexpr (BlockPaths<L1, LMAX, KIND>::list.n > 0) {
-        const int mul = D.mul_in[L1];
-        for (int ub = 0; ub < mul;) {
-            const int left = (mul - ub) / 32;
-            if (MAXC >= 2 && left >= 2) {
-                tp_bwd_block_pair<L1, LMAX, KIND, (MAXC >= 2 ? 2 : 1)>(D, ub + lane, e, v, w, gY, s_w, s_G, x, gm,
-                                                                       gxo);
-                ub += 64;
-            } else {
-                tp_bwd_block_pair<L1, LMAX, KIND, 1>(D, ub + lane, e, v, w, gY, s_w, s_G, x, gm, gxo);
-                ub += 32;
-            }
-        }
-    }
-}
-
-// Phase E of the pair kernel: a warp per pair (slot e: receiver v = s_dst[e],
-// sender w = s_src[e]).
-template <int LMAX, int KIND, int MAXC>
-__device__ __forceinline__ void tp_bwd_chunk_pair(const ConvDesc& D, int ne, const int* s_dst, const int* s_src,
-                                                  float* s_w, const float* s_G, float* s_gY,
-                                                  const float* __restrict__ x, const float* __restrict__ gm,
-                                                  unsigned long long* __restrict__ gx) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int e = warp; e < ne; e += CONV_WARPS) {
-        const int v = s_dst[e], w = s_src[e];
-        constexpr int NYS = LMAX >= 3 ? 16 : 9;
-        float gY[NYS];
-#pragma unroll
-        for (int i = 0; i < NYS; ++i) gY[i] = 0.0f;
-        // l1 = 0 (one component per channel) takes two channels per lane; the
-        // others one (two spill; measured 0.31 ms faster than one everywhere)
-        tp_bwd_l1_pair<0, LMAX, KIND, 2 * MAXC>(D, lane, e, v, w, gY, s_w, s_G, x, gm, gx);
-        tp_bwd_l1_pair<1, LMAX, KIND, MAXC>(D, lane, e, v, w, gY, s_w, s_G, x, gm, gx);
-        if constexpr (LMAX >= 2) tp_bwd_l1_pair<2, LMAX, KIND, MAXC>(D, lane, e, v, w, gY, s_w, s_G, x, gm, gx);
-        if constexpr (LMAX >= 3) tp_bwd_l1_pair<3, LMAX, KIND, MAXC>(D, lane, e, v, w, gY, s_w, s_G, x, gm, gx);
-        constexpr int NY = (LMAX + 1) * (LMAX + 1);
-#pragma unroll
-        for (int i = 0; i < NY; ++i) gY[i] = warp_sum(gY[i]);
-        if (lane < NYS) {
-            float val = 0.0f;
-#pragma unroll
-            for (int i = 0; i < NY; ++i) if (lane == i) val = gY[i];
+            for (int i = 1; i < NY; ++i) if (lane == i) val = gY[i];
             s_gY[e * y_stride<LMAX>() + lane] = val;
         }
     }
@@ -358,23 +262,13 @@ conv_bwd_kernel(const ConvDesc D, const float* __restrict__ W1, const __nv_bfloa
         }
         cp_async_commit();
         chunk_w_gemm<H, BF ? 1 : 3, false>(D, L, smem, W3T_h);
-        // E: per-edge (or per-pair) adjoint of the tensor product (path lists fixed per
-        // block kind); the H = 32 kernels (small models) take one channel per lane
-        constexpr int MAXC = H == 64 ? 2 : 1;
-        if constexpr (PAIR) {      // one channel per lane for l1 >= 1: two directions' operands in registers
-            switch (D.kind) {
-                case 0: tp_bwd_chunk_pair<LMAX, 0, 1>(D, ne, s_dst, s_src, s_w, smem + L.G, s_gY, x, gm, gx); break;
-                case 1: tp_bwd_chunk_pair<LMAX, 1, 1>(D, ne, s_dst, s_src, s_w, smem + L.G, s_gY, x, gm, gx); break;
-                case 2: tp_bwd_chunk_pair<LMAX, 2, 1>(D, ne, s_dst, s_src, s_w, smem + L.G, s_gY, x, gm, gx); break;
-                default: tp_bwd_chunk_pair<LMAX, 3, 1>(D, ne, s_dst, s_src, s_w, smem + L.G, s_gY, x, gm, gx); break;
-            }
-        } else {
-            switch (D.kind) {
-                case 0: tp_bwd_chunk<LMAX, 0, MAXC>(D, ne, s_dst, s_src, s_w, smem + L.G, s_gY, x, gm, gx); break;
-                case 1: tp_bwd_chunk<LMAX, 1, MAXC>(D, ne, s_dst, s_src, s_w, smem + L.G, s_gY, x, gm, gx); break;
-                case 2: tp_bwd_chunk<LMAX, 2, MAXC>(D, ne, s_dst, s_src, s_w, smem + L.G, s_gY, x, gm, gx); break;
-                default: tp_bwd_chunk<LMAX, 3, MAXC>(D, ne, s_dst, s_src, s_w, smem + L.G, s_gY, x, gm, gx); break;
-            }
+        // E: adjoint of the tensor product (path lists fixed per block kind)
+        constexpr int DIRS = PAIR ? 2 : 1;
+        switch (D.kind) {
+            case 0: tp_bwd_chunk<LMAX, 0, DIRS>(D, ne, s_dst, s_src, s_w, smem + L.G, s_gY, x, gm, gx); break;
+            case 1: tp_bwd_chunk<LMAX, 1, DIRS>(D, ne, s_dst, s_src, s_w, smem + L.G, s_gY, x, gm, gx); break;
+            case 2: tp_bwd_chunk<LMAX, 2, DIRS>(D, ne, s_dst, s_src, s_w, smem + L.G, s_gY, x, gm, gx); break;
+            default: tp_bwd_chunk<LMAX, 3, DIRS>(D, ne, s_dst, s_src, s_w, smem + L.G, s_gY, x, gm, gx); break;
         }
         // F: dE/dH2 = dE/dw @ W3^T
         chunk_gw_gemm<H, BF ? (PAIR ? 2 : 1) : 3, BF ? 1 : 3>(D, L, smem, W3_h);

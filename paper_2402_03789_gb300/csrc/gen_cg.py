@@ -14,6 +14,7 @@ For each coupling (l1, l2, l3) with l <= LMAX it writes a specialisation
     CG<l1,l2,l3>::G(Y, G)        G[m1][m3] = sum_m2 C[m1,m2,m3] Y[m2]
     CG<l1,l2,l3>::gY(a, b, gY)   gY[m2] += sum_{m1,m3} C[m1,m2,m3] a[m1] b[m3]
     CG<l1,l2,l3>::M(T, m)        m[m3] = sum_{m1,m2} C[m1,m2,m3] T[m1][m2]
+    CG<l1,l2,l3>::S(S, gY)       gY[m2] += sum_{m1,m3} C[m1,m2,m3] S[m1][m3]
 with every structurally zero coefficient dropped.
 """
 
@@ -153,6 +154,12 @@ def emit(path):
                     terms = [(a, b, v) for (a, b, cc), v in sorted(tab.items()) if cc == c]
                     expr = " + ".join(f"{_lit(v)} * T[{a * (2 * l2 + 1) + b}]" for a, b, v in terms)
                     lines.append(f"    m[{c}] = {expr};")
+                lines.append("  }")
+                lines.append("  static __device__ __forceinline__ void S(const float* __restrict__ s, float* __restrict__ gy) {")
+                for bb in range(2 * l2 + 1):
+                    terms = [(a, c, v) for (a, b2, c), v in sorted(tab.items()) if b2 == bb]
+                    for a, c, v in terms:
+                        lines.append(f"    gy[{bb}] = fmaf({_lit(v)}, s[{a * n3 + c}], gy[{bb}]);")
                 lines.append("  }")
                 lines.append("};")
                 lines.append("")

@@ -305,6 +305,7 @@ struct ConvDesc {
     int32_t mul_in[NL];  // multiplicity of l in the block input (0 = absent)
     int32_t x_off[NL];
     int32_t pbeg[NL], pend[NL];   // paths with l1 = l occupy [pbeg, pend)
+    int32_t gb_off[NL];           // blocked message rows (pair adjoint): first value of l1's blocks
     int32_t kind;               // bit 0: first block (input mul0 x 0e), bit 1: last block (l3 = 0)
     float r_cut;
     float env_a, env_b, env_c;  // envelope coefficients
@@ -335,6 +336,9 @@ struct GemmProb {
     int32_t R, K, N;           // K and N are multiples of 32 (every multiplicity is)
     int32_t lda, a_off, ldc, c_off;
     int32_t accumulate;        // 1: C += A B, 0: C = A B
+    // blocked C rows (null: rows as above): component m of column c goes to
+    // c_blk[c / 32] + 32 m + c % 32
+    const int* c_blk = nullptr;
     // a second product added to the same rows (K2 = 0: none): C = A B + A2 B2
     int32_t K2 = 0, lda2 = 0, a_off2 = 0;
     const float* A2 = nullptr;
@@ -364,6 +368,7 @@ struct LayerDev {
     __nv_bfloat16* mlp1Th = nullptr;  // [3][H][H] W2^T (B operand of H1 @ W2)
     __nv_bfloat16* mlp2h = nullptr;   // [3][W][H] W3^T (N-major for the mma B operand)
     __nv_bfloat16* mlp2Th = nullptr;  // [3][H][W] W3
+    int* g_blk[NL] = {};     // c_blk of dE/dm of degree l (blocked rows)
     float* lin1[NL] = {};  float* lin1T[NL] = {};  __nv_bfloat16* lin1h[NL] = {};  __nv_bfloat16* lin1Th[NL] = {};
     float* sc[NL] = {};    float* scT[NL] = {};    __nv_bfloat16* sch[NL] = {};    __nv_bfloat16* scTh[NL] = {};
     float* lin2[NL] = {};  float* lin2T[NL] = {};  __nv_bfloat16* lin2h[NL] = {};  __nv_bfloat16* lin2Th[NL] = {};

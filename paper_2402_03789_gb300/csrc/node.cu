@@ -110,7 +110,7 @@ gemm_f32_kernel(const __grid_constant__ GemmBatch batch) {
         if (row >= rows) break;
         const int64_t v = row / P.R;
         const int mm = (int)(row % P.R);
-        float* cp = P.C + v * P.ldc + P.c_off + (int64_t)mm * P.N + col;
+        float* cp = P.C + v * P.ldc + (P.c_blk ? P.c_blk[col >> 5] + 32 * mm + (col & 31) : P.c_off + mm * P.N + col);
         float4 o = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
         if (P.accumulate) {
             const float4 c = *reinterpret_cast<const float4*>(cp);
@@ -259,7 +259,7 @@ gemm_bf16_kernel(const __grid_constant__ GemmBatch batch) {
             if (r >= rows) continue;
             const int64_t v = r / P.R;
             const int mm = (int)(r % P.R);
-            float* cp = P.C + v * P.ldc + P.c_off + (int64_t)mm * P.N;
+            float* cp = P.C + v * P.ldc + (P.c_blk ? P.c_blk[nbase >> 5] + 32 * mm - nbase : P.c_off + mm * P.N);
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
                 const int col = nbase + j * 8 + 2 * tq;

@@ -2,7 +2,9 @@
 receiver over groups of four edges) through whole evaluations, against the FP64
 oracle, where its layout can go wrong: receivers without edges, groups with one
 to three empty slots, fewer chunks than helper warps, fewer receivers than CTAs,
-every number of paths and tiles a block kind and degree gives.
+every number of paths and tiles a block kind and degree gives.  The adjoint over
+pairs reads blocked rows of dE/dm and takes the scalars 64 channels at a time with
+a remainder of 32; "odd" has both.
 
 Tolerances: FP32 1e-5 of the forces' norm, as everywhere for that path (sums of
 some thousand products at 2^-24 each); BF16 5e-3 (operands at 2^-9)."""
@@ -18,7 +20,7 @@ pytestmark = pytest.mark.gpu
 
 WIDE = ModelSpec(n_species=3, n_layers=2, mul=(32, 96, 64), avg_num_neigh=34.0)
 SPECS = {"sevennet0": MODEL_SEVENNET0, "l2_32": benchmark_model(3, 32, 2), "l3_32": benchmark_model(3, 32, 3),
-         "uneven": WIDE}
+         "uneven": WIDE, "odd": ModelSpec(n_species=3, n_layers=3, mul=(96, 32, 64), avg_num_neigh=34.0)}
 
 
 def _gas(n, box, seed):
@@ -53,7 +55,7 @@ def test_sparse_receivers(name, prec):
 
 @pytest.mark.parametrize("prec", ["fp32", "bf16"])
 @pytest.mark.parametrize("name,counts", [("sevennet0", {"Si": 2, "O": 3}), ("l2_32", {"Si": 50, "O": 101}),
-                                         ("l3_32", {"Si": 21, "O": 40}), ("uneven", {"N": 31, "O": 60})])
+                                         ("l3_32", {"Si": 21, "O": 40}), ("uneven", {"N": 31, "O": 60}), ("odd", {"Si": 11, "O": 20})])
 def test_dense_cells(name, counts, prec):
     s = random_structure(counts, 2.4, 1.5, seed=11)
     _check(SPECS[name], s.pos, s.cell, s.species, prec)

@@ -100,7 +100,7 @@ __device__ __forceinline__ void tp_bwd_block(const ConvDesc& D, int u0, int e, c
 #pragma unroll
     for (int q = 0; q < DIRS; ++q) {
         if constexpr (DIRS == 2) {               // blocked rows
-            const int lane = threadIdx.x & 31;
+            const int lane = u0 & 31;
             const float* gr = gm + (size_t)recv[q] * D.m_dim + D.gb_off[L1] + (u0 - lane) * NG + lane;
 #pragma unroll
             for (int h = 0; h < NCH; ++h)
@@ -151,7 +151,7 @@ __device__ __forceinline__ void tp_bwd_chunk(const ConvDesc& D, int ne, const in
                                              float* s_w, const float* s_G, float* s_gY,
                                              const float* __restrict__ x, const float* __restrict__ gm,
                                              unsigned long long* __restrict__ gx) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int t = chunk_tid(), lane = t & 31, warp = t >> 5;
     for (int e = warp; e < ne; e += CONV_WARPS) {
         int recv[DIRS], send[DIRS];
         recv[0] = s_dst[e];
@@ -221,18 +221,19 @@ conv_bwd_kernel(const ConvDesc D, const float* __restrict__ W1, const __nv_bfloa
     __syncthreads();
     const int E0 = s_range[0], E1 = s_range[1];
     if (E0 >= E1) return;                        // beyond the device-side unit count
-    const int t = threadIdx.x, warp = t >> 5;
     const int* s_src = reinterpret_cast<const int*>(smem + L.src);
     const int* s_dst = reinterpret_cast<const int*>(smem + L.dst);
     float* s_w = smem + L.w;
     float* s_gY = smem + L.gY;
     load_W1<H>(D, L, smem, W1);
     float* s_gdp = smem + L.gdp;
+    float* s_gB = smem + L.stage;                // [NB][EC] (phase B keeps H1 there)
     // The next chunk's edge records are copied to shared memory asynchronously
     // (thread e < EC copies edge e), so no registers hold them across a chunk.
-    __shared__ float4 s_ngeo[EC];
-    __shared__ int s_nsrc[EC], s_ndst[EC], s_ne[PAIR ? EC : 1], s_ecur[PAIR ? EC : 1];
+    __shared__ float4 s_ngeo[EC], s_pgeo[EC];
+    __shared__ int s_nsrc[EC], s_ndst[EC], s_ne[PAIR ? EC : 1], s_ecur[PAIR ? EC : 1], s_pe[PAIR ? EC : 1];
     auto stage = [&](int c) {
+        const int t = chunk_tid();
         if (t < EC && c + t < E1) {
             cp_async4(reinterpret_cast<float*>(s_nsrc + t), reinterpret_cast<const float*>(src + c + t));
             cp_async4(reinterpret_cast<float*>(s_ndst + t), reinterpret_cast<const float*>(dst + c + t));
@@ -240,20 +241,87 @@ conv_bwd_kernel(const ConvDesc D, const float* __restrict__ W1, const __nv_bfloa
             if constexpr (PAIR) cp_async4(reinterpret_cast<float*>(s_ne + t), reinterpret_cast<const float*>(eidx + c + t));
         }
     };
+    // Phase A of the chunk at c, by 16 threads (i = 0..15), from the staged records
+    auto features = [&](int c, int i) {
+        const int n = min(EC, E1 - c);
+        EdgePrefetch pf;
+        if (i < n) {
+            pf.src = s_nsrc[i];
+            pf.dst = s_ndst[i];
+            pf.geom = s_ngeo[i];
+            if constexpr (PAIR) s_ecur[i] = s_ne[i];
+        }
+        chunk_features<LMAX>(D, L, smem, i, c, n, pf);
+    };
+    // G: dE/dd = (dE/dr) u + (I - u u^T) dE/du / r, thread t < EC the unit c + t
+    auto finish = [&](int c, int t, const float4* geo, const int* pe) {
+        const float4 g = geo[t];
+        const float r = g.w, inv = 1.0f / r;
+        const float ux = g.x * inv, uy = g.y * inv, uz = g.z * inv;
+        float env, denv;
+        envelope(D, r / D.r_cut, env, denv);
+        denv /= D.r_cut;
+        const float th = 3.14159265358979f * r / D.r_cut;
+        const float dth = 3.14159265358979f / D.r_cut;
+        float s1, c1;
+        sincosf(th, &s1, &c1);
+        float sm = 0.0f, sn = s1, cm = 1.0f, cn = c1;
+        const float k2 = 2.0f / D.r_cut;
+        float dEdr = 0.0f;
+        for (int n = 0; n < D.n_basis; ++n) {
+            const float nn = (float)(n + 1);
+            const float f = k2 * sn * inv;
+            const float df = k2 * (nn * dth * cn * inv - sn * inv * inv);
+            dEdr = fmaf(s_gB[n * EC + t], df * env + f * denv, dEdr);
+            const float ns = 2.0f * c1 * sn - sm;
+            const float nc = 2.0f * c1 * cn - cm;
+            sm = sn; sn = ns; cm = cn; cn = nc;
+        }
+        const float* gy = s_gY + t * y_stride<LMAX>();
+        const float s3 = 1.7320508075688772f, s15 = 3.872983346207417f, s5 = 2.23606797749979f;
+        float gux = s3 * gy[3], guy = s3 * gy[1], guz = s3 * gy[2];
+        if (D.lmax >= 2) {
+            gux += s15 * (uy * gy[4] + uz * gy[7] + ux * gy[8]);
+            guy += s15 * (ux * gy[4] + uz * gy[5] - uy * gy[8]);
+            guz += s15 * (uy * gy[5] + ux * gy[7]) + 3.0f * s5 * uz * gy[6];
+        }
+        if constexpr (LMAX >= 3) {   // gradients of the degree-3 polynomials (projected below)
+            const float a3 = 2.0916500663351889f, b3 = 10.246950765959598f;
+            const float c3 = 1.6201851746019651f, d3 = 1.3228756555322954f;
+            const float zz5 = 5.0f * uz * uz - 1.0f;
+            gux += gy[9] * 6.0f * a3 * ux * uy + gy[10] * b3 * uy * uz + gy[13] * c3 * zz5 +
+                   gy[14] * b3 * ux * uz + gy[15] * 3.0f * a3 * (ux * ux - uy * uy);
+            guy += gy[9] * 3.0f * a3 * (ux * ux - uy * uy) + gy[10] * b3 * ux * uz + gy[11] * c3 * zz5 -
+                   gy[14] * b3 * uy * uz - gy[15] * 6.0f * a3 * ux * uy;
+            guz += gy[10] * b3 * ux * uy + gy[11] * 10.0f * c3 * uy * uz +
+                   gy[12] * d3 * (15.0f * uz * uz - 3.0f) + gy[13] * 10.0f * c3 * ux * uz +
+                   gy[14] * 0.5f * b3 * (ux * ux - uy * uy);
+        }
+        const float dot = gux * ux + guy * uy + guz * uz;
+        float* o = gd + (size_t)(PAIR ? pe[t] : c + t) * 3;
+        o[0] = s_gdp[3 * t] + dEdr * ux + (gux - dot * ux) * inv;
+        o[1] = s_gdp[3 * t + 1] + dEdr * uy + (guy - dot * uy) * inv;
+        o[2] = s_gdp[3 * t + 2] + dEdr * uz + (guz - dot * uz) * inv;
+    };
     stage(E0);
     cp_async_commit();
     cp_async_wait_all();
-    for (int c0 = E0; c0 < E1; c0 += EC) {
-        const int ne = min(EC, E1 - c0);
-        __syncthreads();
-        EdgePrefetch cur;
-        if (t < ne) {
-            cur.src = s_nsrc[t];
-            cur.dst = s_ndst[t];
-            cur.geom = s_ngeo[t];
-            if constexpr (PAIR) s_ecur[t] = s_ne[t];      // published by the prologue's barrier
+    // Phases A and G are serial chains of 16 threads, some 2,500 cycles each.  BF16: the
+    // first warp runs G of the previous chunk while the second runs A of this one
+    // (24,000 atoms, adjoints of 5 layers 12.25 -> 11.9 ms).  FP32, where the other CTA's
+    // W3 products fill the SM meanwhile: one after the other (3,000 atoms: 3.55 ms an
+    // evaluation, 3.59 ms overlapped).  Results are the same bits either way.
+    constexpr bool OVERLAP = BF;
+    for (int c0 = E0;; c0 += EC) {
+        const int t = chunk_tid(), warp = t >> 5;
+        __syncthreads();       // the previous chunk's dE/dbasis and dE/dY; this chunk's records
+        if constexpr (OVERLAP) {
+            if (c0 > E0 && t < EC && c0 - EC + t < E1) finish(c0 - EC, t, s_pgeo, s_pe);
         }
-        chunk_prologue<H, BF, LMAX>(D, L, smem, c0, ne, cur, W2T_h);
+        if (c0 >= E1) break;
+        if (const int i = OVERLAP ? t - 32 : t; i >= 0 && i < EC) features(c0, i);
+        const int ne = min(EC, E1 - c0);
+        __syncthreads();       // phase A of this chunk
         stage(c0 + EC);        // lands by the wait before phase G
         // dE/dd of the blocks done so far, copied to shared memory for phase G
         if (t < 3 * ne) {
@@ -261,6 +329,7 @@ conv_bwd_kernel(const ConvDesc D, const float* __restrict__ W1, const __nv_bfloa
             else cp_async4(s_gdp + t, gd + (size_t)c0 * 3 + t);
         }
         cp_async_commit();
+        chunk_hidden<H, BF, LMAX>(D, L, smem, W2T_h);
         chunk_w_gemm<H, BF ? 1 : 3, false>(D, L, smem, W3T_h);
         // E: adjoint of the tensor product (path lists fixed per block kind)
         constexpr int DIRS = PAIR ? 2 : 1;
@@ -270,26 +339,20 @@ conv_bwd_kernel(const ConvDesc D, const float* __restrict__ W1, const __nv_bfloa
             case 2: tp_bwd_chunk<LMAX, 2, DIRS>(D, ne, s_dst, s_src, s_w, smem + L.G, s_gY, x, gm, gx); break;
             default: tp_bwd_chunk<LMAX, 3, DIRS>(D, ne, s_dst, s_src, s_w, smem + L.G, s_gY, x, gm, gx); break;
         }
-        // F: dE/dH2 = dE/dw @ W3^T
+        // F: gA2 = (dE/dw @ W3^T) * silu'(A2), then gH1 = gA2 @ W2^T; gA1 = gH1 * silu'(A1); gB = gA1 @ W1^T
         chunk_gw_gemm<H, BF ? (PAIR ? 2 : 1) : 3, BF ? 1 : 3>(D, L, smem, W3_h);
-        // MLP adjoint: gA2 = gH2 * silu'(A2); gH1 = gA2 @ W2^T; gA1 = gH1 * silu'(A1); gB = gA1 @ W1^T
         float* s_gH = smem + L.gH;
         float* s_A1 = smem + L.A1;
         float* s_A2 = smem + L.A2;
-        for (int i = t; i < H * EC; i += CONV_THREADS) s_gH[i] *= dsiluf_(s_A2[i]);
-        __syncthreads();
         {   // gA1 = (gA2 @ W2^T) * silu'(A1), stored over A2
             constexpr int AT = BF ? (PAIR ? 2 : 1) : 3, BT = BF ? 2 : 3;
             const int lane = t & 31, g = lane >> 2, tq = lane & 3;
-            float c[4] = {0.f, 0.f, 0.f, 0.f};
+            float c[4];
             const int nt = warp;
             if (nt < H / 8) {
                 HiddenB<H, BT> hb;
                 hidden_load<H, BT>(W2_h, nt, hb);
                 hidden_mma<H, AT, BT>(s_gH, hb, c);
-            }
-            __syncthreads();       // every read of A2 (the silu' above) is done
-            if (nt < H / 8) {
                 const int k = nt * 8 + 2 * tq;
                 const int o[4] = {hk<H>(k, g), hk<H>(k + 1, g), hk<H>(k, g + 8), hk<H>(k + 1, g + 8)};
 #pragma unroll
@@ -297,7 +360,6 @@ conv_bwd_kernel(const ConvDesc D, const float* __restrict__ W1, const __nv_bfloa
             }
         }
         __syncthreads();
-        float* s_gB = smem + L.stage;              // [NB][EC]
         for (int i = t; i < D.n_basis * EC; i += CONV_THREADS) {
             const int n = i / EC, e = i % EC;
             float a = 0.0f;
@@ -305,57 +367,16 @@ conv_bwd_kernel(const ConvDesc D, const float* __restrict__ W1, const __nv_bfloa
             for (int k = 0; k < H; ++k) a = fmaf(s_A2[hk<H>(k, e)], smem[L.W1 + n * H + k], a);
             s_gB[i] = a;
         }
+        if constexpr (OVERLAP) {
+            if (t < EC) {          // for phase G (read by the same thread)
+                s_pgeo[t] = reinterpret_cast<const float4*>(smem + L.geo)[t];
+                if constexpr (PAIR) s_pe[t] = s_ecur[t];
+            }
+        }
         cp_async_wait_all();
-        __syncthreads();
-        // G: dE/dd = (dE/dr) u + (I - u u^T) dE/du / r
-        if (t < ne) {
-            const float4 g = reinterpret_cast<const float4*>(smem + L.geo)[t];
-            const float r = g.w, inv = 1.0f / r;
-            const float ux = g.x * inv, uy = g.y * inv, uz = g.z * inv;
-            float env, denv;
-            envelope(D, r / D.r_cut, env, denv);
-            denv /= D.r_cut;
-            const float th = 3.14159265358979f * r / D.r_cut;
-            const float dth = 3.14159265358979f / D.r_cut;
-            float s1, c1;
-            sincosf(th, &s1, &c1);
-            float sm = 0.0f, sn = s1, cm = 1.0f, cn = c1;
-            const float k2 = 2.0f / D.r_cut;
-            float dEdr = 0.0f;
-            for (int n = 0; n < D.n_basis; ++n) {
-                const float nn = (float)(n + 1);
-                const float f = k2 * sn * inv;
-                const float df = k2 * (nn * dth * cn * inv - sn * inv * inv);
-                dEdr = fmaf(s_gB[n * EC + t], df * env + f * denv, dEdr);
-                const float ns = 2.0f * c1 * sn - sm;
-                const float nc = 2.0f * c1 * cn - cm;
-                sm = sn; sn = ns; cm = cn; cn = nc;
-            }
-            const float* gy = s_gY + t * y_stride<LMAX>();
-            const float s3 = 1.7320508075688772f, s15 = 3.872983346207417f, s5 = 2.23606797749979f;
-            float gux = s3 * gy[3], guy = s3 * gy[1], guz = s3 * gy[2];
-            if (D.lmax >= 2) {
-                gux += s15 * (uy * gy[4] + uz * gy[7] + ux * gy[8]);
-                guy += s15 * (ux * gy[4] + uz * gy[5] - uy * gy[8]);
-                guz += s15 * (uy * gy[5] + ux * gy[7]) + 3.0f * s5 * uz * gy[6];
-            }
-            if constexpr (LMAX >= 3) {   // gradients of the degree-3 polynomials (projected below)
-                const float a3 = 2.0916500663351889f, b3 = 10.246950765959598f;
-                const float c3 = 1.6201851746019651f, d3 = 1.3228756555322954f;
-                const float zz5 = 5.0f * uz * uz - 1.0f;
-                gux += gy[9] * 6.0f * a3 * ux * uy + gy[10] * b3 * uy * uz + gy[13] * c3 * zz5 +
-                       gy[14] * b3 * ux * uz + gy[15] * 3.0f * a3 * (ux * ux - uy * uy);
-                guy += gy[9] * 3.0f * a3 * (ux * ux - uy * uy) + gy[10] * b3 * ux * uz + gy[11] * c3 * zz5 -
-                       gy[14] * b3 * uy * uz - gy[15] * 6.0f * a3 * ux * uy;
-                guz += gy[10] * b3 * ux * uy + gy[11] * 10.0f * c3 * uy * uz +
-                       gy[12] * d3 * (15.0f * uz * uz - 3.0f) + gy[13] * 10.0f * c3 * ux * uz +
-                       gy[14] * 0.5f * b3 * (ux * ux - uy * uy);
-            }
-            const float dot = gux * ux + guy * uy + guz * uz;
-            float* o = gd + (size_t)(PAIR ? s_ecur[t] : c0 + t) * 3;
-            o[0] = s_gdp[3 * t] + dEdr * ux + (gux - dot * ux) * inv;
-            o[1] = s_gdp[3 * t + 1] + dEdr * uy + (guy - dot * uy) * inv;
-            o[2] = s_gdp[3 * t + 2] + dEdr * uz + (guz - dot * uz) * inv;
+        if constexpr (!OVERLAP) {
+            __syncthreads();
+            if (t < ne) finish(c0, t, reinterpret_cast<const float4*>(smem + L.geo), s_ecur);
         }
     }
 }

@@ -263,6 +263,15 @@ __device__ __forceinline__ void bf16_terms(float x, float y, uint32_t (&t)[NT]) 
     }
 }
 
+// threadIdx.x for one chunk: opaque, so that the addresses made from it are not kept in
+// registers across the adjoint's chunks (its BF16 kernel fills 128 a thread, and what
+// spills leaves the small L1: 24,000 atoms, adjoints 12.23 ms without, 11.9 ms with it).
+__device__ __forceinline__ int chunk_tid() {
+    int t = threadIdx.x;
+    asm volatile("" : "+r"(t));
+    return t;
+}
+
 __device__ __forceinline__ void mma_bf16(float* c, const uint32_t* a, const uint32_t* b) {
     asm volatile(
         "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
@@ -355,7 +364,7 @@ __device__ __forceinline__ void chunk_w_gemm(const ConvDesc& D, const ConvSmem& 
     __syncthreads();
 }
 
-// Phase F: gH2[k][e] = sum_c gw[e][c] W3[c][k]; A operand dE/dw in AT terms, B
+// Phase F: gA2[k][e] = silu'(A2[k][e]) sum_c gw[e][c] W3[c][k]; A operand dE/dw in AT terms, B
 // operand W3 in BT terms of [H][W].
 // K (the W columns, in blocks of 32) is split between four groups of two warps;
 // within a group each warp owns H/16 n tiles of 8 hidden units for the group's
@@ -434,7 +443,7 @@ __device__ __forceinline__ void chunk_gw_gemm(const ConvDesc& D, const ConvSmem&
     }
     __syncthreads();
     for (int i = t; i < H * EC; i += CONV_THREADS)
-        s_gH[i] = ((s_gH[i] + s_w[i]) + s_w[H * EC + i]) + s_w[2 * H * EC + i];
+        s_gH[i] = (((s_gH[i] + s_w[i]) + s_w[H * EC + i]) + s_w[2 * H * EC + i]) * dsiluf_(smem[L.A2 + i]);
     __syncthreads();
 }
 
@@ -495,7 +504,6 @@ __device__ __forceinline__ void hidden_mma(const float* __restrict__ s_in, const
     }
 }
 
-// Phases A-C shared by both kernels.  Leaves s_src/s_dst/Y/B/A1/A2/H2/G filled.
 // Edge data of one chunk, fetched one chunk ahead by threads 0..EC-1.
 struct EdgePrefetch {
     int src = 0, dst = -1, first = 0;           // first: index of the receiver's first edge
@@ -521,31 +529,39 @@ __device__ __forceinline__ void load_W1(const ConvDesc& D, const ConvSmem& L, fl
     for (int i = threadIdx.x; i < D.n_basis * H; i += CONV_THREADS) smem[L.W1 + i] = W1[i];
 }
 
-template <int H, bool BF, int LMAX>
-__device__ __forceinline__ void chunk_prologue(const ConvDesc& D, const ConvSmem& L, float* smem,
-                                               int c0, int ne, const EdgePrefetch& pf,
-                                               const __nv_bfloat16* __restrict__ W2T_h) {
-    const int t = threadIdx.x, warp = t >> 5;
+// Phase A: edge records, harmonics and basis of a chunk, thread i < EC edge i
+// (published by the next barrier).
+template <int LMAX>
+__device__ __forceinline__ void chunk_features(const ConvDesc& D, const ConvSmem& L, float* smem, int i,
+                                               int c0, int ne, const EdgePrefetch& pf) {
     int* s_src = reinterpret_cast<int*>(smem + L.src);
     int* s_dst = reinterpret_cast<int*>(smem + L.dst);
     float* s_Y = smem + L.Y;
     float* s_B = smem + L.B;       // [NB][EC]
-    if (t < EC) {
-        if (t < ne) {
-            s_src[t] = pf.src;
-            s_dst[t] = pf.dst;
-            reinterpret_cast<int*>(smem + L.first)[t] = pf.first >= c0;   // receiver starts here
-            reinterpret_cast<float4*>(smem + L.geo)[t] = pf.geom;
-            edge_features<LMAX>(D, pf.geom, s_Y + t * y_stride<LMAX>(), s_B + t, EC);
-        } else {
-            s_src[t] = 0;
-            s_dst[t] = -1;
-            reinterpret_cast<float4*>(smem + L.geo)[t] = make_float4(0.f, 0.f, 0.f, 1.f);
-            for (int i = 0; i < y_stride<LMAX>(); ++i) s_Y[t * y_stride<LMAX>() + i] = 0.0f;
-            for (int n = 0; n < D.n_basis; ++n) s_B[n * EC + t] = 0.0f;
-        }
+    if (i < ne) {
+        s_src[i] = pf.src;
+        s_dst[i] = pf.dst;
+        reinterpret_cast<int*>(smem + L.first)[i] = pf.first >= c0;   // receiver starts here
+        reinterpret_cast<float4*>(smem + L.geo)[i] = pf.geom;
+        edge_features<LMAX>(D, pf.geom, s_Y + i * y_stride<LMAX>(), s_B + i, EC);
+    } else {
+        s_src[i] = 0;
+        s_dst[i] = -1;
+        reinterpret_cast<float4*>(smem + L.geo)[i] = make_float4(0.f, 0.f, 0.f, 1.f);
+        for (int n = 0; n < y_stride<LMAX>(); ++n) s_Y[i * y_stride<LMAX>() + n] = 0.0f;
+        for (int n = 0; n < D.n_basis; ++n) s_B[n * EC + i] = 0.0f;
     }
-    __syncthreads();
+}
+
+// Phases B and C.  Leaves A1/A2/H2/G filled.
+template <int H, bool BF, int LMAX>
+__device__ __forceinline__ void chunk_hidden(const ConvDesc& D, const ConvSmem& L, float* smem,
+                                             const __nv_bfloat16* __restrict__ W2T_h) {
+    const int t = threadIdx.x, warp = t >> 5;
+    float* s_Y = smem + L.Y;
+    float* s_B = smem + L.B;       // [NB][EC]
+    constexpr int AT = BF ? 1 : 3, BT = BF ? 2 : 3;
+    HiddenB<H, BT> hb;
     // B: A1 = B @ W1 (layout [H][EC]); H1 = silu(A1) lives in the staging area until
     // phase D.  Thread (j, edge group): hidden unit j for EPT consecutive edges.
     float* s_A1 = smem + L.A1;
@@ -582,9 +598,7 @@ __device__ __forceinline__ void chunk_prologue(const ConvDesc& D, const ConvSmem
     __syncthreads();
     if (warp < H / 8) {          // A2 = H1 @ W2, H2 = silu(A2)
         const int lane = t & 31, g = lane >> 2, tq = lane & 3, nt = warp;
-        constexpr int AT = BF ? 1 : 3, BT = BF ? 2 : 3;
         float c[4];
-        HiddenB<H, BT> hb;
         hidden_load<H, BT>(W2T_h, nt, hb);
         hidden_mma<H, AT, BT>(s_H1, hb, c);
         const int j = nt * 8 + 2 * tq;

@@ -208,7 +208,9 @@ conv_fwd_kernel(const ConvDesc D, const float* __restrict__ W1, const __nv_bfloa
     for (int c0 = E0; c0 < E1; c0 += EC) {
         const int ne = min(EC, E1 - c0);
         __syncthreads();
-        chunk_prologue<H, BF, LMAX>(D, L, smem, c0, ne, pf, W2T_h);
+        if (threadIdx.x < EC) chunk_features<LMAX>(D, L, smem, threadIdx.x, c0, ne, pf);
+        __syncthreads();
+        chunk_hidden<H, BF, LMAX>(D, L, smem, W2T_h);
         pf.fetch(c0 + EC, E1, dst, src, geom, row_ptr);   // next chunk's edges, in flight meanwhile
         chunk_w_gemm<H, BF ? 1 : 3, BF>(D, L, smem, W3T_h);
         switch (D.kind) {

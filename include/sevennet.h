@@ -189,8 +189,8 @@ sevennet_status sevennet_eval_energy_forces_virial(sevennet_model* model, int64_
  * once with more room if the device reported more edges than the capacity.
  * Results are bit-for-bit repeatable; in FP32 a structure's results are the
  * same bits alone and in any batch, in BF16 they agree to BF16 rounding (the
- * tensor-core forward groups a receiver's edges from chunk boundaries that
- * move with the batch). */
+ * forward of models with a 32-wide radial MLP groups a receiver's edges from
+ * chunk boundaries that move with the batch). */
 sevennet_status sevennet_eval_batch_dev(sevennet_model* model, int32_t n_structs,
                                         const int64_t* atom_offsets, const double* cells,
                                         const int32_t* pbc, const int32_t* species_dev,
@@ -326,7 +326,7 @@ void sevennet_md_destroy(sevennet_md* md);
 /* Serving: continuous batching of independent structures.  Requests are
  * copied at submission.  At creation the HBM budget is split evenly over
  * n_streams slots and each slot's workspace and pinned buffers are allocated
- * for the atoms its share holds (about 47 KB per atom for SevenNet-0), so
+ * for the atoms its share holds (about 51 KB per atom for SevenNet-0), so
  * running a batch allocates and frees nothing and waits for nothing on the
  * host.  A worker thread packs queued requests into a free slot (up to
  * max_batch_structs structures and the slot's atoms), enqueues copy-in,

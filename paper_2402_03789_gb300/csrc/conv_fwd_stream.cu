@@ -25,6 +25,11 @@
 // (the units of a CTA type run different code; with the loop unrolled over two
 // groups and three copies of the epilogue the instruction cache missed and the
 // l1 = 2 type ran twice as long).
+//
+// Measured on the middle block of 128x0e+64x1e+32x2e, 24,000 atoms, BF16: 0.70 ms and
+// 0.09 ms of radial.cu, against 2.01 ms of the chunked kernel (conv_fwd_tc.cu); FP32,
+// 3,000 atoms, whole evaluation 8.26 -> 5.7 ms.  Bound by the consumers' FP32 lanes
+// and, for units of l1 = 0 (the fewest multiply-adds per byte of a row), by the row copies.
 #include "conv_common.cuh"
 #include "packed_fma.cuh"
 #include "tmem.cuh"

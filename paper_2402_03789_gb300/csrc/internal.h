@@ -457,7 +457,7 @@ struct Workspace {
     float* h = nullptr;           // [N][h_max]
     float* xs = nullptr;          // [T][N][x_max]
     float* ys = nullptr;          // [T][N][y_max]
-    float* m = nullptr;           // [N][m_max] (messages, then their gradients)
+    float* m = nullptr;           // [N][m_max] messages, then their gradients (blocked rows for the adjoint over pairs)
     float* gy = nullptr;          // [N][y_max]
     float* gx = nullptr;          // [N][x_max]
     unsigned long long* gxq = nullptr;   // [N][x_max] fixed-point sums of dE/dx

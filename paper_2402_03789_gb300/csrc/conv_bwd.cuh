@@ -406,8 +406,11 @@ sevennet_status conv_configure_bwd_mode(int H, size_t need) {
 }
 
 // bound: an upper bound on the number of units (the count itself is *count, on
-// the device).  Tiles of 1..4 chunks, at least about 8 waves of tiles where the
-// input allows (4 measured fastest on the 24,000-atom cell: 2 and 8 were slower).
+// the device; in an evaluation about half of it).  Tiles of 1..4 chunks (24,000
+// atoms: 4 measured fastest, 3 and 6 1 % slower).  FP32: at least 16 waves of tiles by
+// the bound, so that the last wave is a small part (8 waves: 1,500 atoms degree 3
+// 2.23 against 2.11 ms, 3,000 atoms 3.54 against 3.52).  BF16: 8, because its chunks
+// overlap inside a tile (16 waves: 2,777 atoms, one convolution, 0.821 against 0.806 ms).
 template <bool PAIR>
 void conv_bwd_dispatch(const LayerDev& L, int H, bool bf, int64_t bound, const int* count, const int* dst,
                        const int* src, const float4* geom, const int* eidx, const float* x, const float* gm,
@@ -415,7 +418,7 @@ void conv_bwd_dispatch(const LayerDev& L, int H, bool bf, int64_t bound, const i
     const int lm = L.conv.lmax;
     bound = std::max<int64_t>(bound, 0);
     const int64_t wave = (int64_t)conv_grid(INT64_MAX, conv_ctas_per_sm(lm));
-    const int tile = EC * (int)std::min<int64_t>(4, std::max<int64_t>(1, bound / (EC * 8 * wave)));
+    const int tile = EC * (int)std::min<int64_t>(4, std::max<int64_t>(1, bound / (EC * (bf ? 8 : 16) * wave)));
     const int grid = (int)std::max<int64_t>(1, (bound + tile - 1) / tile);
     const size_t sm = smem_bytes(L.conv, H, true, bf);
 #define SN_LB(HH, BB, LL) conv_bwd_kernel<HH, BB, LL, PAIR><<<grid, CONV_THREADS, sm, st>>>(           \

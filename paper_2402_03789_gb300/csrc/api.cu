@@ -639,7 +639,7 @@ void model_layer_forward(sevennet_model* M, Workspace* ws, int t, int64_t N, int
         const int64_t cap = (ws->cap_edges + 1) / 2;
         launch_radial(L, prec, cap, ws->pair_ptr + N, ws->p_geom, ws->grad, st);
         launch_conv_fwd_stream(L, prec, N, cap, ws->row_ptr, ws->quad_ptr, ws->quads, ws->src, ws->geom,
-                               reinterpret_cast<const int*>(ws->gd), ws->grad, x, ws->m, ws->flags, st);
+                               reinterpret_cast<const int*>(ws->gd), ws->grad, x, ws->m, ws->flags, M->wait_limit, st);
     } else {
         launch_conv_fwd(L, M->H, prec, N, E, ws->row_ptr, ws->dst, ws->src, ws->geom, x, ws->m, st, ws->flags);
     }
@@ -1395,6 +1395,9 @@ sevennet_status sevennet_profile_read(sevennet_model* M, int32_t n_max, char* na
     if (n_out) *n_out = n;
     return SEVENNET_OK;
 }
+
+// Not part of the interface: lets a test make the streaming forward's waits run out.
+void sn_test_set_wait_limit(sevennet_model* M, uint32_t cycles) { M->wait_limit = cycles; }
 
 int64_t sevennet_launch_count(void) { return g_launch_count.load(); }
 

@@ -82,6 +82,7 @@ struct StArgs {                      // launch-wide pointers
     const float* x;
     float* m;
     int* flags;
+    unsigned wait_limit;             // clock cycles
 };
 
 struct StCtx {                       // one CTA's stream
@@ -163,6 +164,7 @@ __device__ __forceinline__ void st_unit(const StType& T, const StUnit& U, const 
             for (int c = 0; c < N3; ++c) mp[c * m_mul[i]] = out[c];
         });
     };
+    auto wait = [&](uint64_t* bar, unsigned phase) { return pipe_wait(bar, phase, C.abort, A.wait_limit); };
     const unsigned tm0 = C.tmem_w + ((unsigned)(32 * r) << 16);
     int cur = -1, s = -1, d = -1, c0 = C.Q0 - ST_E / 4, vq = -1;
     unsigned parity = 0, wparity = 0, mine = 0, tm = 0;
@@ -181,7 +183,7 @@ __device__ __forceinline__ void st_unit(const StType& T, const StUnit& U, const 
             c0 += ST_E / 4;
             if (++s == C.stages) { s = 0; parity ^= 1u; }
             if (++d == C.w_bufs) { d = 0; wparity ^= 1u; }
-            end = c0 >= C.Q1 || !pipe_wait(C.full + s, parity, C.abort) || !pipe_wait(C.wfull + d, wparity, C.abort);
+            end = c0 >= C.Q1 || !wait(C.full + s, parity) || !wait(C.wfull + d, wparity);
             if (end) break;
             tc_fence_after();
             s_y = reinterpret_cast<const float*>(C.sm + C.L.y) + s * NY * ST_E;
@@ -267,6 +269,7 @@ template <int LMAX, bool BF>
 __device__ __forceinline__ void st_helper(const StType& T, const StArgs& A, const StCtx& C, int wh) {
     constexpr int SPL = BF ? 1 : 3, NY = (LMAX + 1) * (LMAX + 1) - 1, NH2 = BF ? 1 : 2;
     const int lane = threadIdx.x & 31;
+    auto wait = [&](uint64_t* bar, unsigned phase) { return pipe_wait(bar, phase, C.abort, A.wait_limit); };
     const unsigned idesc = umma_idesc(128, ST_E);
     const int n_chunks = (C.Q1 - C.Q0 + ST_E / 4 - 1) / (ST_E / 4);
     const int nh = C.helpers;
@@ -293,7 +296,7 @@ __device__ __forceinline__ void st_helper(const StType& T, const StArgs& A, cons
 #pragma unroll
             for (int k = 0; k < NH2; ++k) hv[q][k] = __ldg(g + k);
         }
-        if (!pipe_wait(C.empty + s, par, C.abort)) break;
+        if (!wait(C.empty + s, par)) break;
         // x rows by bulk copies, a lane a row; zeros in the empty slots
         const int row_bytes = T.row_floats * 4;
         unsigned char* xs = C.sm + C.L.x + s * C.L.x_stage;
@@ -319,7 +322,7 @@ __device__ __forceinline__ void st_helper(const StType& T, const StArgs& A, cons
         if ((lane & 3) == 0) reinterpret_cast<int*>(C.sm + C.L.dst)[s * (ST_E / 4) + (lane >> 2)] = v;
         __syncwarp();
         if (lane == 0) mbar_arrive(C.full + s);
-        if (round > 0 && !pipe_wait(C.bdone + wh, (round - 1) & 1u, C.abort)) break;    // this helper's B tile is free
+        if (round > 0 && !wait(C.bdone + wh, (round - 1) & 1u)) break;    // this helper's B tile is free
         unsigned char* bt = C.sm + C.L.b + wh * SPL * ST_B_BYTES;
 #pragma unroll
         for (int q = 0; q < 8; ++q) {
@@ -347,8 +350,8 @@ __device__ __forceinline__ void st_helper(const StType& T, const StArgs& A, cons
             }
         }
         asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
-        if (j > 0 && !pipe_wait(C.turn + wh, (wh == 0 ? round - 1 : round) & 1u, C.abort)) break;
-        if (!pipe_wait(C.wempty + d, wpar, C.abort)) break;
+        if (j > 0 && !wait(C.turn + wh, (wh == 0 ? round - 1 : round) & 1u)) break;
+        if (!wait(C.wempty + d, wpar)) break;
         tc_fence_after();
         __syncwarp();
         if (elect_one()) {
@@ -376,7 +379,7 @@ __device__ __forceinline__ void st_helper(const StType& T, const StArgs& A, cons
         for (s += nh; s >= C.stages; s -= C.stages) par ^= 1u;
         for (d += nh; d >= C.w_bufs; d -= C.w_bufs) wpar ^= 1u;
     }
-    if (round > 0) pipe_wait(C.bdone + wh, (round - 1) & 1u, C.abort);    // no MMA in flight when TMEM is freed
+    if (round > 0) wait(C.bdone + wh, (round - 1) & 1u);    // no MMA in flight when TMEM is freed
 }
 
 // First v in [0, n] with row_ptr[v] >= key; one whole warp.
@@ -721,11 +724,11 @@ int64_t st_grad_bytes(const sevennet_model* M) {
 void launch_conv_fwd_stream(const LayerDev& Ld, sevennet_precision prec, int64_t n_atoms, int64_t cap_pairs,
                             const int* row_ptr, const int* quad_ptr, const int2* quads, const int* src,
                             const float4* geom, const int* pair_of, const void* h2, const float* x, float* m, int* flags,
-                            cudaStream_t st) {
+                            unsigned wait_limit, cudaStream_t st) {
     const bool bf = prec == SEVENNET_BF16;
     const StPlan& P = Ld.st[bf ? 1 : 0];
     if (n_atoms <= 0) return;
-    const StArgs A{(int)n_atoms, Ld.conv.x_dim, Ld.conv.m_dim, cap_pairs, row_ptr, quad_ptr, src, pair_of, quads, geom, h2, x, m, flags};
+    const StArgs A{(int)n_atoms, Ld.conv.x_dim, Ld.conv.m_dim, cap_pairs, row_ptr, quad_ptr, src, pair_of, quads, geom, h2, x, m, flags, wait_limit};
 #define SN_ST_RUN(LL, KK, BB)                                                             \
     if (Ld.conv.lmax == LL && Ld.conv.kind == KK && bf == BB) {                           \
         conv_fwd_stream_kernel<LL, KK, BB><<<P.n_cta, ST_THREADS, P.smem, st>>>(P, A);    \

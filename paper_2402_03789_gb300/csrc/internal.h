@@ -400,6 +400,7 @@ struct sevennet_model {
     int T = 0, lmax = 0, H = 0, NB = 0;
     int h_max = 0, x_max = 0, y_max = 0, m_max = 0;
     int h2_bytes = 0;           // hidden activations per pair for the streaming forward (0: not used)
+    unsigned wait_limit = 4000000000u;   // cycles that a wait of the streaming forward may take (about two seconds)
     std::vector<sn::LayerDev> layers;
     float* embed = nullptr;     // [n_species][mul0]
     float* readout = nullptr;   // [mul0] = scale * R0 R1 / sqrt(mul0 hid)
@@ -575,7 +576,7 @@ sevennet_status st_configure(int lmax);
 void launch_conv_fwd_stream(const LayerDev& L, sevennet_precision prec, int64_t n_atoms, int64_t cap_pairs,
                             const int* row_ptr, const int* quad_ptr, const int2* quads, const int* src,
                             const float4* geom, const int* pair_of, const void* h2, const float* x, float* m,
-                            int* flags, cudaStream_t st);
+                            int* flags, unsigned wait_limit, cudaStream_t st);
 void launch_quads(int64_t n_atoms, const int* row_ptr, const int* quad_ptr, int2* quads, cudaStream_t st);
 void launch_radial(const LayerDev& L, sevennet_precision prec, int64_t cap_pairs, const int* n_pairs,
                    const float4* p_geom, void* h2, cudaStream_t st);

@@ -85,22 +85,26 @@ __device__ __forceinline__ void mbar_add_tx(uint64_t* bar, unsigned bytes) {
                  : "memory");
 }
 
-// Bounded wait of a pipeline: false when the limit ran out here or another
-// thread of the CTA gave up (*abort).
-__device__ __forceinline__ bool pipe_wait(uint64_t* bar, unsigned parity, volatile int* abort) {
+// Bounded wait of a whole warp on a pipeline's barrier: false when `limit` clock cycles
+// (at most about two seconds; 0: the phase is not over yet) ran out here or another thread
+// of the CTA gave up (*abort).  The verdict is a vote: lanes that read the barrier and the
+// flag at different times must not part, since full-warp shuffles and votes follow.
+__device__ __forceinline__ bool pipe_wait(uint64_t* bar, unsigned parity, volatile int* abort, unsigned limit) {
     const unsigned a = smem_u32(bar);
-    long long t0 = 0;
+    unsigned done;
+    asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                 " selp.u32 %0, 1, 0, p;\n}\n" : "=r"(done) : "r"(a), "r"(parity) : "memory");
+    if (__all_sync(0xffffffffu, done)) return true;
+    const long long t0 = clock64();
     while (true) {
-        unsigned done;
-        // the last operand lets the hardware suspend the warp for up to that many ns
-        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
-                     " selp.u32 %0, 1, 0, p;\n}\n" : "=r"(done) : "r"(a), "r"(parity), "r"(20000u) : "memory");
-        if (done) return true;
-        if (t0 == 0) t0 = clock64();
-        else if (*abort || clock64() - t0 > BULK_WAIT_LIMIT) {
+        if (__any_sync(0xffffffffu, *abort || clock64() - t0 >= (long long)limit)) {
             *abort = 1;
             return false;
         }
+        // the last operand lets the hardware suspend the warp for up to that many ns
+        asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
+                     " selp.u32 %0, 1, 0, p;\n}\n" : "=r"(done) : "r"(a), "r"(parity), "r"(20000u) : "memory");
+        if (__all_sync(0xffffffffu, done)) return true;
     }
 }
 

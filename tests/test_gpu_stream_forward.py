@@ -9,6 +9,8 @@ a remainder of 32; "odd" has both.
 Tolerances: FP32 1e-5 of the forces' norm, as everywhere for that path (sums of
 some thousand products at 2^-24 each); BF16 5e-3 (operands at 2^-9)."""
 
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -67,3 +69,26 @@ def test_single_atom_and_isolated_atoms():
     for pos in (np.zeros((1, 3)), np.array([[0.0, 0, 0], [15.0, 15, 15]])):
         E, F, W = get_model(spec).evaluate(pos, cell, np.zeros(len(pos), np.int32), precision="bf16")
         assert np.isfinite(E) and np.abs(F).max() == 0 and np.abs(W).max() == 0
+
+
+def _set_wait_limit(model, cycles):
+    model.lib.sn_test_set_wait_limit(model.handle, ctypes.c_uint32(cycles))
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+def test_waits_that_run_out_end_the_call(prec):
+    """With no time for any wait, the first one that is not over at once gives up: every
+    warp must leave its pipeline together and the call report it (status ETIMEDOUT), and
+    the tensor memory must be free for the next call, which gives the same bits as before."""
+    s = random_structure({"N": 31, "O": 60}, 2.4, 1.5, seed=11)
+    model = get_model(WIDE)
+    before = model.evaluate(s.pos, s.cell, s.species, precision=prec)
+    try:
+        _set_wait_limit(model, 0)
+        with pytest.raises(RuntimeError) as err:
+            model.evaluate(s.pos, s.cell, s.species, precision=prec)
+        assert err.value.status == -5
+    finally:
+        _set_wait_limit(model, 4000000000)
+    after = model.evaluate(s.pos, s.cell, s.species, precision=prec)
+    assert after[0] == before[0] and np.array_equal(after[1], before[1]) and np.array_equal(after[2], before[2])

@@ -1113,11 +1113,12 @@ sevennet_status eval_enqueue(sevennet_model* M, Workspace* ws, const BatchHost& 
 sevennet_status check_flags(const int* f) {
     SN_CHECK(f[1] == 0, SEVENNET_EINVAL, "two atoms closer than 1e-8 A");
     SN_CHECK(f[3] == 0, SEVENNET_EINVAL, "species index out of range");
+    // before the overflow that the NaN messages of a timeout bring about in the adjoint
+    SN_CHECK(f[FLAG_COPY_TIMEOUT] == 0, SEVENNET_ETIMEDOUT, "a wait of the forward convolution ran out");
     SN_CHECK(f[FLAG_GX_OVERFLOW] == 0, SEVENNET_EOVERFLOW,
              "a feature gradient in the convolution adjoint reached 2^16 (outside the fixed-point range)");
     SN_CHECK(f[FLAG_EDGE_OVERFLOW] == 0, SEVENNET_EOVERFLOW, "neighbour list larger than its capacity");
     SN_CHECK(f[2] == 0, SEVENNET_ECUDA, "internal error: inconsistent neighbour list (a reverse edge not found, or a stored Verlet list entry out of range)");
-    SN_CHECK(f[FLAG_COPY_TIMEOUT] == 0, SEVENNET_ETIMEDOUT, "a bulk copy did not complete within its bounded wait");
     return SEVENNET_OK;
 }
 

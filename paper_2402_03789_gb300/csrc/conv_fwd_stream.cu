@@ -92,6 +92,7 @@ struct StCtx {                       // one CTA's stream
     unsigned tmem, tmem_w;           // A tiles, weight buffers
     uint64_t *full, *empty, *wfull, *wempty, *turn, *bdone;
     volatile int* abort;
+    int* issued;                     // per helper: twice its chunks whose MMAs are issued, plus one for row copies ahead of them
 };
 
 // A group of up to four consecutive edges of one receiver: x = first edge,
@@ -280,6 +281,7 @@ __device__ __forceinline__ void st_helper(const StType& T, const StArgs& A, cons
     int2 quad = fetch_quad(wh);
     int s = wh % C.stages, d = wh % C.w_bufs;
     unsigned round = 0;
+    int ahead = 0;                             // 1: row copies of a chunk whose MMAs are not issued
     unsigned par = 1u ^ ((wh / C.stages) & 1u), wpar = 1u ^ ((wh / C.w_bufs) & 1u);   // empty: the first round passes
     for (int j = wh; j < n_chunks; j += nh) {
         const int e = quad.x + min(lane & 3, quad_last(quad));
@@ -297,6 +299,7 @@ __device__ __forceinline__ void st_helper(const StType& T, const StArgs& A, cons
             for (int k = 0; k < NH2; ++k) hv[q][k] = __ldg(g + k);
         }
         if (!wait(C.empty + s, par)) break;
+        ahead = 1;
         // x rows by bulk copies, a lane a row; zeros in the empty slots
         const int row_bytes = T.row_floats * 4;
         unsigned char* xs = C.sm + C.L.x + s * C.L.x_stage;
@@ -376,10 +379,30 @@ __device__ __forceinline__ void st_helper(const StType& T, const StArgs& A, cons
         }
         __syncwarp();
         ++round;
+        ahead = 0;
         for (s += nh; s >= C.stages; s -= C.stages) par ^= 1u;
         for (d += nh; d >= C.w_bufs; d -= C.w_bufs) wpar ^= 1u;
     }
-    if (round > 0) wait(C.bdone + wh, (round - 1) & 1u);    // no MMA in flight when TMEM is freed
+    if (lane == 0) C.issued[wh] = 2 * (int)round + ahead;
+    // no MMA in flight when TMEM is freed, whether or not a wait ran out
+    if (round > 0 && !wait(C.bdone + wh, (round - 1) & 1u)) mbar_wait(C.bdone + wh, (round - 1) & 1u, BULK_WAIT_LIMIT);
+}
+
+// After a wait ran out, one thread: waits until the last chunk that went through each of
+// the n barriers is complete (ahead 0: its MMAs, 1: its row copies).  Chunk j belongs to
+// helper j mod nh and uses phase j / n of barrier j mod n; a barrier's chunks are issued in order.
+__device__ __noinline__ void st_drain(uint64_t* bars, int n, int nh, const int* issued, int ahead) {
+    int top = -1;
+    for (int w = 0; w < nh; ++w) {
+        const int done = (issued[w] + ahead) / 2;
+        if (done > 0) top = max(top, w + (done - 1) * nh);
+    }
+    for (int b = 0; b < n; ++b)
+        for (int j = top; j >= 0; --j)
+            if (j % n == b && j / nh < (issued[j % nh] + ahead) / 2) {
+                mbar_wait(bars + b, (j / n) & 1, BULK_WAIT_LIMIT / 8);
+                break;
+            }
 }
 
 // First v in [0, n] with row_ptr[v] >= key; one whole warp.
@@ -418,8 +441,9 @@ conv_fwd_stream_kernel(const __grid_constant__ StPlan P, const StArgs A) {
     C.wempty = C.wfull + ST_MAX_W;
     C.turn = C.wempty + ST_MAX_W;
     C.bdone = C.turn + ST_NH;
-    int* misc = reinterpret_cast<int*>(C.sm + C.L.misc);       // [0] abort, [1] tmem, [2..3] receiver range
+    int* misc = reinterpret_cast<int*>(C.sm + C.L.misc);       // [0] abort, [1] tmem, [2..3] receiver range, [4..7] issued
     C.abort = misc;
+    C.issued = misc + 4;
     const int nb = T.n_cta, b = (int)blockIdx.x - T.cta0;
     if (warp == 0) {
         const long long n_e = A.quad_ptr[A.n_atoms];
@@ -441,6 +465,7 @@ conv_fwd_stream_kernel(const __grid_constant__ StPlan P, const StArgs A) {
                 mbar_init(C.wempty + d, T.n_units * ST_NQ);
             }
             for (int w = 0; w < ST_NH; ++w) {
+                C.issued[w] = 0;
                 mbar_init(C.turn + w, 1);
                 mbar_init(C.bdone + w, 1);
             }
@@ -505,16 +530,17 @@ conv_fwd_stream_kernel(const __grid_constant__ StPlan P, const StArgs A) {
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    if (misc[0] && threadIdx.x == 0) {         // a wait ran out: let what is in flight end, then report
-        for (int d = 0; d < C.w_bufs; ++d) {
-            mbar_wait(C.wfull + d, 0, BULK_WAIT_LIMIT / 8);
-            mbar_wait(C.wfull + d, 1, BULK_WAIT_LIMIT / 8);
+    if (misc[0]) {             // a wait ran out: what is in flight ends, the CTA's messages are NaN, and the call reports it
+        if (threadIdx.x == 0) {
+            st_drain(C.wfull, C.w_bufs, C.helpers, C.issued, 0);
+            st_drain(C.full, C.stages, C.helpers, C.issued, 1);
+            if (A.flags) atomicOr(A.flags + FLAG_COPY_TIMEOUT, 1);
         }
-        for (int s = 0; s < P.stages; ++s) {
-            mbar_wait(C.full + s, 0, BULK_WAIT_LIMIT / 8);
-            mbar_wait(C.full + s, 1, BULK_WAIT_LIMIT / 8);
-        }
-        if (A.flags) atomicOr(A.flags + FLAG_COPY_TIMEOUT, 1);
+        for (int v = v0 + warp; v < v1; v += ST_THREADS / 32)
+            for (int r = 0; r < T.n_units; ++r)
+                for (int i = 0; i < T.u[r].n_paths; ++i)
+                    for (int c = 0; c < T.u[r].n3[i]; ++c)
+                        A.m[(size_t)v * A.m_dim + T.u[r].m_off[i] + c * T.u[r].m_mul[i] + lane] = __int_as_float(0x7fc00000);
     }
     __syncthreads();
     if (warp == 3) tmem_dealloc(C.tmem, 512);

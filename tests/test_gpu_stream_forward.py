@@ -13,8 +13,10 @@ import ctypes
 
 import numpy as np
 import pytest
+import torch
 
 import oracle
+from paper_2402_03789_gb300 import _lib
 from synth import ModelSpec, MODEL_SEVENNET0, benchmark_model, random_structure
 from gpu_common import errors, get_model
 
@@ -87,8 +89,29 @@ def test_waits_that_run_out_end_the_call(prec):
         _set_wait_limit(model, 0)
         with pytest.raises(RuntimeError) as err:
             model.evaluate(s.pos, s.cell, s.species, precision=prec)
-        assert err.value.status == -5
+        assert err.value.status == _lib.ETIMEDOUT
     finally:
         _set_wait_limit(model, 4000000000)
     after = model.evaluate(s.pos, s.cell, s.species, precision=prec)
     assert after[0] == before[0] and np.array_equal(after[1], before[1]) and np.array_equal(after[2], before[2])
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+def test_messages_of_a_timed_out_forward_are_nan(prec):
+    """A block whose waits ran out hands on NaN, not partial sums or what an earlier call
+    left: the energy on the device is NaN, and the status is still the timeout's."""
+    s = random_structure({"N": 31, "O": 60}, 2.4, 1.5, seed=11)
+    model = get_model(WIDE)
+    pos = torch.tensor(s.pos, dtype=torch.float64, device="cuda")
+    args = ([0, s.n_atoms], s.cell[None], torch.tensor(s.species, dtype=torch.int32, device="cuda"), pos, prec)
+    out = model.evaluate_batch_dev(*args)
+    assert all(torch.isfinite(t).all() for t in out)
+    try:
+        _set_wait_limit(model, 0)
+        with pytest.raises(RuntimeError) as err:
+            model.evaluate_batch_dev(*args, out=out)
+    finally:
+        _set_wait_limit(model, 4000000000)
+    torch.cuda.synchronize()
+    assert err.value.status == _lib.ETIMEDOUT
+    assert torch.isnan(out[0]).all()

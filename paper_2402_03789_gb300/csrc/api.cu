@@ -493,7 +493,10 @@ static sevennet_status ws_alloc(Workspace* ws, T** p, int64_t count) {
     return SEVENNET_OK;
 }
 
-// Grows the workspace to the given sizes.  Nothing happens (and nothing waits)
+int ws_h2_bytes(const sevennet_model* M, const Workspace* ws) { return std::min(M->h2_bytes, ws->h2_max); }
+
+// Grows the workspace to the given sizes (the server's bytes_per_atom counts what an atom
+// takes here).  Nothing happens (and nothing waits)
 // when the capacities suffice; a reallocation frees the old buffer first, and
 // cudaFree waits for the work that may still use it.
 sevennet_status ws_reserve(sevennet_model* M, Workspace* ws, int64_t n_atoms, int64_t n_edges,
@@ -543,7 +546,7 @@ sevennet_status ws_reserve(sevennet_model* M, Workspace* ws, int64_t n_atoms, in
         SN_TRY(ws_alloc(ws, &ws->gd, E * 3));
         ws->cap_edges = E;
     }
-    const int64_t grad = std::max<int64_t>(ws->cap_atoms * st_grad_bytes(M), (ws->cap_edges + 1) / 2 * M->h2_bytes);
+    const int64_t grad = std::max<int64_t>(ws->cap_atoms * st_grad_bytes(M), (ws->cap_edges + 1) / 2 * ws_h2_bytes(M, ws));
     if (grad > ws->grad_bytes) {
         ws->grad_bytes = 0;
         SN_TRY(ws_alloc(ws, &ws->grad, grad));
@@ -634,7 +637,7 @@ void model_layer_forward(sevennet_model* M, Workspace* ws, int t, int64_t N, int
     }
     run_gemm(M, g, prec, st);
     prof_begin(P, PF_CONV_FWD, st, &ev);
-    const bool stream = pairs && M->h2_bytes >= (prec == SEVENNET_BF16 ? 128 : 256);
+    const bool stream = pairs && ws_h2_bytes(M, ws) >= (prec == SEVENNET_BF16 ? 128 : 256);
     if (stream) {
         const int64_t cap = (ws->cap_edges + 1) / 2;
         launch_radial(L, prec, cap, ws->pair_ptr + N, ws->p_geom, ws->grad, st);

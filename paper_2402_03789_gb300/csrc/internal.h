@@ -455,6 +455,7 @@ struct Workspace {
     // the pairs' hidden activations there while a convolution runs (all five are dead then)
     unsigned char* grad = nullptr;
     int64_t grad_bytes = 0;
+    int h2_max = 256;             // room for hidden activations per pair (128: BF16 evaluations only)
     float* h = nullptr;           // [N][h_max]
     float* xs = nullptr;          // [T][N][x_max]
     float* ys = nullptr;          // [T][N][y_max]
@@ -572,6 +573,7 @@ sevennet_status st_plan_build(sevennet_model* M, LayerDev& L);
 sevennet_status radial_pack(sevennet_model* M, LayerDev& L);
 int st_h2_bytes(const sevennet_model* M);
 int64_t st_grad_bytes(const sevennet_model* M);     // gradients (and h) of one atom
+int ws_h2_bytes(const sevennet_model* M, const Workspace* ws);   // hidden activations per pair in the gradient block
 sevennet_status st_configure(int lmax);
 void launch_conv_fwd_stream(const LayerDev& L, sevennet_precision prec, int64_t n_atoms, int64_t cap_pairs,
                             const int* row_ptr, const int* quad_ptr, const int2* quads, const int* src,

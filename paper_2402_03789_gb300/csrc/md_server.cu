@@ -545,18 +545,23 @@ static double srv_now(const sevennet_server* s) {
     return std::chrono::duration<double>(std::chrono::steady_clock::now() - s->t0).count();
 }
 
-// Device bytes per atom of a slot's workspace: the activations of every block,
-// the messages and gradients, the fixed-point dE/dx sums, and 64 edges.
-static size_t bytes_per_atom(const sevennet_model* M) {
-    const size_t act = (size_t)(M->T * (M->x_max + M->y_max) + M->m_max + M->y_max + M->x_max + 2 * M->h_max) *
-                           sizeof(float) + (size_t)M->x_max * sizeof(unsigned long long) + 200;
-    // dst, src, rev, the clamp's row entries, shift, geometry, dE/dd; the pair list (edge, dst, src, geometry)
-    const size_t per_edge = 4 * 4 + 12 + 16 + 12 + 3 * 4 + 16;
-    return act + per_edge * 64;
+// Device bytes per atom of a slot: what ws_reserve takes for an atom with 64 edges (32
+// pairs, up to 17 groups of four edges) and the slot's own input and output buffers.
+static size_t bytes_per_atom(const sevennet_model* M, const Workspace* ws) {
+    const size_t h2 = (size_t)ws_h2_bytes(M, ws);
+    const size_t act = (size_t)(M->T * (M->x_max + M->y_max) + M->m_max) * sizeof(float);
+    const size_t grad = std::max<size_t>((size_t)st_grad_bytes(M), 32 * h2);
+    // 9 integers, positions and images, sums, 3 bin arrays; positions, forces, species of the slot
+    const size_t per_atom = 9 * 4 + 24 + 12 + 16 + 8 + 72 + 24 + 1 + 3 * 4 + 24 + 24 + 4 + (h2 ? 17 * sizeof(int2) : 0);
+    // dst, src, rev, shift, geometry, dE/dd; the pair list (edge, dst, src, geometry)
+    const size_t per_edge = 3 * 4 + 12 + 16 + 12 + 3 * 4 + 16;
+    return act + grad + per_atom + per_edge * 64;
 }
 
 // Predicted device bytes of one request (its share of a slot's workspace).
-static size_t predict_bytes(const sevennet_model* M, int64_t n) { return bytes_per_atom(M) * (size_t)n + 4096; }
+static size_t predict_bytes(const sevennet_server* S, int64_t n) {
+    return bytes_per_atom(S->M, S->slots[0].ws) * (size_t)n + 4096;
+}
 
 // A slot's workspace and pinned buffers are allocated once, at server creation,
 // for cap_atoms atoms (its share of the HBM budget), so that running a batch
@@ -741,9 +746,10 @@ sevennet_status sevennet_server_create(sevennet_model* M, size_t hbm_budget_byte
             return SEVENNET_ECUDA;
         }
         sl.ws = new Workspace();
+        if (prec == SEVENNET_BF16) sl.ws->h2_max = 128;
     }
     // each slot owns an equal share of the budget, allocated now
-    S->slot_atoms = (int64_t)((hbm_budget_bytes / (size_t)n_streams) / bytes_per_atom(M));
+    S->slot_atoms = (int64_t)((hbm_budget_bytes / (size_t)n_streams) / bytes_per_atom(M, S->slots[0].ws));
     for (auto& sl : S->slots) {
         const sevennet_status s = slot_alloc(M, sl, S->slot_atoms, max_batch_structs);
         if (s != SEVENNET_OK) {
@@ -769,7 +775,7 @@ sevennet_status sevennet_server_submit(sevennet_server* S, const sevennet_reques
     r.species.assign(req->species, req->species + req->n_atoms);
     r.pos.assign(req->pos, req->pos + 3 * req->n_atoms);
     std::copy(req->cell, req->cell + 9, r.cell);
-    r.bytes = predict_bytes(S->M, r.n);
+    r.bytes = predict_bytes(S, r.n);
     SN_CHECK(r.n <= S->slot_atoms, SEVENNET_ENOMEM_ADMIT,
              "request of %lld atoms needs %zu bytes; a slot holds %lld atoms (its share of the %zu-byte budget)",
              (long long)r.n, r.bytes, (long long)S->slot_atoms, S->budget);

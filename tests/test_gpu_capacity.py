@@ -10,7 +10,7 @@ import numpy as np
 import pytest
 
 import oracle
-from synth import MODEL_SEVENNET0, normal_weights, random_structure
+from synth import MODEL_SEVENNET0, benchmark_model, normal_weights, random_structure
 from gpu_common import errors
 
 pytestmark = pytest.mark.gpu
@@ -54,3 +54,23 @@ def test_server_reruns_a_batch_beyond_its_slot_capacity():
     assert r["energy"] == E and np.array_equal(r["forces"], F) and np.array_equal(r["virial"], W)
     srv.close()
     model.close()
+
+
+@pytest.mark.parametrize("prec", ["fp32", "bf16"])
+def test_server_memory_stays_within_its_budget(prec):
+    """The slots' allocations against the budget, for a model whose rows of gradients
+    (7,168 bytes an atom) are smaller than the FP32 hidden activations of 32 pairs that
+    share their memory (8,192).  Each of the about 45 allocations of a slot may round up to 2 MiB."""
+    import torch
+    import paper_2402_03789_gb300 as sn
+    spec = benchmark_model(5, 32, 2)
+    model = sn.SevenNet(spec, normal_weights(oracle.n_params(spec)))
+    s = random_structure({"Si": 20, "O": 40}, 2.2, 1.6, seed=31)
+    model.evaluate(s.pos, s.cell, s.species, prec)            # its own workspace and kernels
+    budget, slots = 12 << 30, 2
+    free = torch.cuda.mem_get_info()[0]
+    srv = sn.Server(model, hbm_budget_bytes=budget, n_streams=slots, max_batch_structs=32, precision=prec)
+    used = free - torch.cuda.mem_get_info()[0]
+    srv.close()
+    model.close()
+    assert 0.97 * budget <= used <= budget + slots * 45 * (2 << 20)

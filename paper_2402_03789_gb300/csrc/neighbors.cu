@@ -191,6 +191,22 @@ __global__ void gather_kernel(int64_t n, int S, const int64_t* __restrict__ atom
     bin_s[i] = bin_of[o];
 }
 
+// (float)sqrt(r2) to the bit, mostly without the FP64 root (it took most of the build's
+// second pass): the FP32 root rt plus (r2 - rt^2) / (2 rt).  That sum is within 2^-45 of
+// the root; where it comes so close to the middle of two floats that this (or the rounding
+// of the FP64 root) could decide, about one edge in 10^5, and at powers of two, where the
+// spacing changes, the FP64 root decides.
+__device__ __forceinline__ float edge_length(double r2) {
+    const float rt = sqrtf((float)r2);
+    const float corr = __fmul_rn((float)fma(-(double)rt, (double)rt, r2), 0.5f / rt);
+    const float c = __fadd_rn(rt, corr);
+    const unsigned bits = __float_as_uint(c);
+    const float half = 0.5f * (__uint_as_float(bits + 1) - c);
+    const float off = __fadd_rn(__fadd_rn(rt, -c), corr);      // what rounding to c left, exact
+    const bool sure = fabsf(off) < half * (1.0f - 0x1p-18f) && (bits & 0x7fffffu) != 0;
+    return sure ? c : (float)sqrt(r2);
+}
+
 // Count (FILL = false) or write (FILL = true) the edges of every internal atom
 // v, a warp per receiver.  The lanes look up the bins within the search range, 32
 // at a time; the members of those bins then form one list in bin order, member
@@ -269,11 +285,7 @@ edges_kernel(int64_t n, double rc2, float rc32, int64_t cap, const int* __restri
                 shift[slot * 3 + 0] = sx - fl_s[w * 3 + 0] + flv[0];
                 shift[slot * 3 + 1] = sy - fl_s[w * 3 + 1] + flv[1];
                 shift[slot * 3 + 2] = sz - fl_s[w * 3 + 2] + flv[2];
-                // |d|: an FP32 root corrected by its FP64 remainder (right to the last bit but
-                // for near ties; the FP64 root took most of the pass)
-                const float rt = sqrtf((float)r2);
-                geom[slot] = make_float4((float)dd[0], (float)dd[1], (float)dd[2],
-                                         fmaf((float)fma(-(double)rt, (double)rt, r2), 0.5f / rt, rt));
+                geom[slot] = make_float4((float)dd[0], (float)dd[1], (float)dd[2], edge_length(r2));
             }
         } else {
             if (hit && r2 < 1e-16) close = true;
@@ -599,7 +611,7 @@ refresh_kernel(int64_t n, double rc2, int64_t cap, const int* __restrict__ perm,
                     shift[slot * 3 + 0] = s0;
                     shift[slot * 3 + 1] = s1;
                     shift[slot * 3 + 2] = s2;
-                    geom[slot] = make_float4((float)dd[0], (float)dd[1], (float)dd[2], (float)sqrt(r2));
+                    geom[slot] = make_float4((float)dd[0], (float)dd[1], (float)dd[2], edge_length(r2));
                 }
             }
         }

@@ -168,3 +168,24 @@ def test_skin_rejects_negative():
     with pytest.raises(sn.SevenNetError):
         md.set_nose_hoover(-5.0, 10.0)
     md.close()
+
+
+def test_built_and_refreshed_lists_have_the_same_distances():
+    """Pairs whose |d| lies next to the middle of two FP32 values, where an inexact root
+    rounds the wrong way: a list built for r_c and one refreshed from a list with a skin
+    must give the same bits, so the same energy."""
+    sn, s, spec, w, model = _tiny(1.0)
+    rng = np.random.default_rng(4)
+    cell = np.eye(3) * 40.0
+    for k in (-4, -2, -1, 1, 2, 4) * 4:
+        c = np.float32(rng.uniform(1.1, 3.9))
+        mid = 0.5 * (np.float64(c) + np.float64(np.nextafter(c, np.float32(9))))
+        pos = np.array([[0.0, 0, 0], [mid * (1 + k * 2.0 ** -52), 0, 0]])
+        sp = np.array([1, 2], np.int32)
+        E, _, _ = model.evaluate(pos, cell, sp, "fp32")
+        md = sn.MD(model, pos, np.zeros((2, 3)), sp, MASSES, cell, "fp32")
+        md.set_skin(0.5)
+        ep, _ = md.step(1, 1e-30)                  # the positions stay as they are
+        md.close()
+        assert ep[0] == E
+    model.close()

@@ -187,10 +187,12 @@ sevennet_status sevennet_eval_energy_forces_virial(sevennet_model* model, int64_
  * (edge arrays preallocated at 64 per atom or the largest count seen); the
  * call synchronises once, at its end, to read the status words, and reruns
  * once with more room if the device reported more edges than the capacity.
- * Results are bit-for-bit repeatable; in FP32 a structure's results are the
- * same bits alone and in any batch, in BF16 they agree to BF16 rounding (the
- * forward of models with a 32-wide radial MLP groups a receiver's edges from
- * chunk boundaries that move with the batch). */
+ * Results are bit-for-bit repeatable; a structure's results are the same bits
+ * alone and in any batch in FP32, and in BF16 where the forward streams edges
+ * (SevenNet-0 among them).  Models that keep the chunked BF16 forward (a 32-wide
+ * radial MLP, or rows of gradients below 4,096 bytes an atom, such as 32x0e+32x1e)
+ * group a receiver's edges from chunk boundaries that move with the batch; there
+ * the results agree to FP32 rounding carried through the BF16 operands. */
 sevennet_status sevennet_eval_batch_dev(sevennet_model* model, int32_t n_structs,
                                         const int64_t* atom_offsets, const double* cells,
                                         const int32_t* pbc, const int32_t* species_dev,
@@ -333,8 +335,8 @@ void sevennet_md_destroy(sevennet_md* md);
  * neighbour build, evaluation and copy-out on the slot's stream, and retires
  * batches by event; batches overlap on the GPU and new arrivals join the next
  * batch without waiting for the running ones.  The results of a structure do
- * not depend on the batch it ran in beyond FP summation order (bit-identical in
- * FP32). */
+ * not depend on the batch it ran in beyond FP summation order (bit-identical
+ * in FP32; in BF16 as for sevennet_eval_batch_dev). */
 typedef struct {
     int64_t        n_atoms;
     const int32_t* species;   /* host [n_atoms] */

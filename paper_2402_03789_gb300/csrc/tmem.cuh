@@ -1,5 +1,5 @@
-// tcgen05 pieces: tensor-memory allocation, the BF16 MMA with both operands in
-// 128-byte-swizzled K-major shared memory, and reads of the accumulator.
+// tcgen05 pieces: tensor-memory allocation, the BF16 MMA with A in tensor memory and
+// B in 128-byte-swizzled K-major shared memory, stores of A and reads of the accumulator.
 #pragma once
 
 #include <cstdint>

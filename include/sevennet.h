@@ -191,8 +191,9 @@ sevennet_status sevennet_eval_energy_forces_virial(sevennet_model* model, int64_
  * alone and in any batch in FP32, and in BF16 where the forward streams edges
  * (SevenNet-0 among them).  Models that keep the chunked BF16 forward (a 32-wide
  * radial MLP, rows of gradients below 4,096 bytes an atom, such as 32x0e+32x1e, or
- * blocks whose channels do not fit the streaming kernel's shared memory) group a receiver's edges from chunk boundaries that move with the batch; there
- * the results agree to FP32 rounding carried through the BF16 operands. */
+ * blocks whose channels do not fit the streaming kernel's shared memory) group a
+ * receiver's edges from chunk boundaries that move with the batch; there the
+ * results agree to FP32 rounding carried through the BF16 operands. */
 sevennet_status sevennet_eval_batch_dev(sevennet_model* model, int32_t n_structs,
                                         const int64_t* atom_offsets, const double* cells,
                                         const int32_t* pbc, const int32_t* species_dev,

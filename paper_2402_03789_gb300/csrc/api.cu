@@ -286,6 +286,13 @@ static sevennet_status dev_upload(sevennet_model* M, const std::vector<T>& h, T*
     return SEVENNET_OK;
 }
 
+// Gives a device array back before the model is destroyed (waits for the work that reads it).
+template <typename T>
+static void dev_release(sevennet_model* M, T* p) {
+    M->allocations.erase(std::remove(M->allocations.begin(), M->allocations.end(), (void*)p), M->allocations.end());
+    cudaFree(p);
+}
+
 static std::vector<float> scaled(const double* w, int rows, int cols, double s, bool transpose) {
     std::vector<float> o((size_t)rows * cols);
     for (int i = 0; i < rows; ++i)
@@ -1013,18 +1020,20 @@ sevennet_status sevennet_create_model(const sevennet_model_config* cfg, const do
             auto w2 = scaled(weights + e2->off, H, D.W, s2, false);
             auto w2T = scaled(weights + e2->off, H, D.W, s2, true);
             auto w1T = scaled(weights + e1->off, H, H, 1.0 / std::sqrt((double)H), true);
-            float *w1_dev = nullptr, *w2_dev = nullptr;
+            // FP32 on the device only until the BF16 terms and fragments are made
+            float *w1_dev = nullptr, *w1T_dev = nullptr, *w2_dev = nullptr, *w2T_dev = nullptr;
             if ((s = dev_upload(M, w0, &L.mlp0))) return fail(s);
             if ((s = dev_upload(M, w1, &w1_dev))) return fail(s);
-            if ((s = dev_upload(M, w1T, &L.mlp1T))) return fail(s);
+            if ((s = dev_upload(M, w1T, &w1T_dev))) return fail(s);
             if ((s = dev_upload(M, w2, &w2_dev))) return fail(s);
-            if ((s = dev_upload(M, w2T, &L.mlp2T))) return fail(s);
+            if ((s = dev_upload(M, w2T, &w2T_dev))) return fail(s);
             if ((s = dev_terms(M, w1_dev, w1.size(), &L.mlp1h))) return fail(s);     // [k][j]
-            if ((s = dev_terms(M, L.mlp1T, w1.size(), &L.mlp1Th))) return fail(s);   // [j][k]
-            if ((s = dev_terms(M, L.mlp2T, w2.size(), &L.mlp2h))) return fail(s);    // [W][H]
+            if ((s = dev_terms(M, w1T_dev, w1.size(), &L.mlp1Th))) return fail(s);  // [j][k]
+            if ((s = dev_terms(M, w2T_dev, w2.size(), &L.mlp2h))) return fail(s);    // [W][H]
             if ((s = dev_terms(M, w2_dev, w2.size(), &L.mlp2Th))) return fail(s);    // [H][W]
-            if ((s = radial_pack(M, L))) return fail(s);
-            if ((s = st_plan_build(M, L))) return fail(s);
+            if ((s = radial_pack(M, L, w1T_dev))) return fail(s);
+            if ((s = st_plan_build(M, L, w2T_dev))) return fail(s);
+            for (float* p : {w1_dev, w1T_dev, w2_dev, w2T_dev}) dev_release(M, p);
         }
     }
     sevennet_status s = conv_configure(H, M->layers);

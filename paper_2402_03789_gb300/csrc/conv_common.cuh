@@ -49,16 +49,6 @@ __device__ __forceinline__ int hk(int k, int e) {
     return ((k >> 1) << 5) | ((((k & 1) << 4) | e) ^ (t << 3));
 }
 
-// Inverse of hk: the (k, e) stored at position i.
-template <int H>
-__device__ __forceinline__ void hk_inv(int i, int& k, int& e) {
-    const int line = i >> 5;
-    const int t = ((line * 8 / H) + line) & 3;         // 4 k / H with k = 2 line (H / 4 is even)
-    const int p = (i & 31) ^ (t << 3);
-    k = 2 * line + (p >> 4);
-    e = p & 15;
-}
-
 // The staging region holds H1 and dE/dbasis.  dE/dH2 (adjoint) reuses H2, which is
 // dead once phase D has run.  The BF16 kernels stay under 97 KB so two CTAs leave
 // about 60 KB of each SM's 256 KB to the L1 cache.

@@ -629,7 +629,6 @@ static void st_plan_types(const ConvDesc& D, const std::vector<StU>& units, int 
                 StUnit& V = T.u[q];
                 V.l1 = (int16_t)u.l1;
                 V.set = (int16_t)u.set;
-                V.group = (int16_t)u.g;
                 V.n_paths = (int16_t)S.cnt[u.set];
                 T.tiles = std::max(T.tiles, V.n_paths);
                 for (int k = 0; k < T.n_seg; ++k)
@@ -685,7 +684,7 @@ static void st_plan_types(const ConvDesc& D, const std::vector<StU>& units, int 
     }
 }
 
-sevennet_status st_plan_build(sevennet_model* M, LayerDev& L) {
+sevennet_status st_plan_build(sevennet_model* M, LayerDev& L, const float* W3T) {
     using U = StU;
     const ConvDesc& D = L.conv;
     L.st[0].ok = L.st[1].ok = 0;
@@ -707,6 +706,7 @@ sevennet_status st_plan_build(sevennet_model* M, LayerDev& L) {
         if (n_types < 1 || n_types > ST_MAX_TYPES || sms < n_types) return SEVENNET_OK;
         st_plan_types(D, units, sms, L.st);
     }
+    if (!L.st[0].ok && !L.st[1].ok) return SEVENNET_OK;
     const int n_types = L.st[0].n_types;
     // W3 as the A operand: row 32 r + lane of tile i = path i of unit r; three BF16
     // terms, of which the BF16 path reads the first
@@ -728,7 +728,7 @@ sevennet_status st_plan_build(sevennet_model* M, LayerDev& L) {
             return SEVENNET_ENOMEM;
         }
         M->allocations.push_back(p);
-        st_pack_kernel<<<tiles * 32, 256>>>(rows, tiles, L.mlp2T, static_cast<__nv_bfloat16*>(p));
+        st_pack_kernel<<<tiles * 32, 256>>>(rows, tiles, W3T, static_cast<__nv_bfloat16*>(p));
         L.st[0].t[t].w3 = L.st[1].t[t].w3 = p;
     }
     SN_CUDA(cudaGetLastError());

@@ -12,7 +12,6 @@ include/sevennet.h:
 
 For each coupling (l1, l2, l3) with l <= LMAX it writes a specialisation
     CG<l1,l2,l3>::G(Y, G)        G[m1][m3] = sum_m2 C[m1,m2,m3] Y[m2]
-    CG<l1,l2,l3>::gY(a, b, gY)   gY[m2] += sum_{m1,m3} C[m1,m2,m3] a[m1] b[m3]
     CG<l1,l2,l3>::M(T, m)        m[m3] = sum_{m1,m2} C[m1,m2,m3] T[m1][m2]
     CG<l1,l2,l3>::S(S, gY)       gY[m2] += sum_{m1,m3} C[m1,m2,m3] S[m1][m3]
 with every structurally zero coefficient dropped.
@@ -141,13 +140,6 @@ def emit(path):
                         else:
                             expr = " + ".join(f"{_lit(v)} * Y[{b}]" for b, v in terms)
                         lines.append(f"    g[{a * n3 + c}] = {expr};")
-                lines.append("  }")
-                lines.append("  static __device__ __forceinline__ void gY(const float* __restrict__ a, const float* __restrict__ b, float* __restrict__ gy) {")
-                for bb in range(2 * l2 + 1):
-                    terms = [(a, c, v) for (a, b2, c), v in sorted(tab.items()) if b2 == bb]
-                    if terms:
-                        expr = " + ".join(f"{_lit(v)} * (a[{a}] * b[{c}])" for a, c, v in terms)
-                        lines.append(f"    gy[{bb}] += {expr};")
                 lines.append("  }")
                 lines.append("  static __device__ __forceinline__ void M(const float* __restrict__ T, float* __restrict__ m) {")
                 for c in range(n3):

@@ -257,7 +257,7 @@ __host__ __device__ constexpr int st_set_cost(int l1, int lmax, int kind, int j)
 // 128 TMEM lanes), the W3 rows they need as the MMA's A operand, and the pieces
 // of an x row they read.
 struct StUnit {
-    int16_t l1, set, group, n_paths;
+    int16_t l1, set, n_paths;
     int32_t xoff, xstep;                 // floats: first channel in a staged x row, step between components
     int16_t n3[4];                       // 2 l3 + 1 of each path
     int32_t m_off[ST_TILES], m_mul[ST_TILES];   // message row: first channel of each path, step between components
@@ -360,8 +360,6 @@ struct LayerDev {
     bool last;
     // device weights, pre-scaled by 1/sqrt(fan_in) (and 1/avg_num_neigh for mlp2)
     float* mlp0 = nullptr;   // [NB][H]
-    float* mlp1T = nullptr;  // [H][H] W2^T
-    float* mlp2T = nullptr;  // [W][H]
     uint2* mlp1F = nullptr;  // W2 as B fragments, three BF16 terms (radial.cu)
     // three BF16 terms each (the BF16 path reads the first, of W2 the first two)
     __nv_bfloat16* mlp1h = nullptr;   // [3][H][H] W2 as stored (B operand of gA2 @ W2^T)
@@ -569,8 +567,8 @@ void launch_conv_fwd_tc(const LayerDev& L, int H, int64_t n_atoms, int64_t n_edg
 // Streaming forward over a symmetric list with its pairs (conv_fwd_stream.cu).
 // h2: hidden activations of the radial MLP per pair (launch_radial), 64 values a
 // pair: FP32, or BF16 in the BF16 path; pair_of: the pair of every edge.
-sevennet_status st_plan_build(sevennet_model* M, LayerDev& L);
-sevennet_status radial_pack(sevennet_model* M, LayerDev& L);
+sevennet_status st_plan_build(sevennet_model* M, LayerDev& L, const float* W3T);
+sevennet_status radial_pack(sevennet_model* M, LayerDev& L, const float* W2T);
 int st_h2_bytes(const sevennet_model* M);
 int64_t st_grad_bytes(const sevennet_model* M);     // gradients (and h) of one atom
 int ws_h2_bytes(const sevennet_model* M, const Workspace* ws);   // hidden activations per pair in the gradient block

@@ -38,7 +38,7 @@ __global__ void radial_pack_kernel(const float* __restrict__ W2T, uint2* __restr
     }
 }
 
-sevennet_status radial_pack(sevennet_model* M, LayerDev& L) {
+sevennet_status radial_pack(sevennet_model* M, LayerDev& L, const float* W2T) {
     if (M->H != 64) return SEVENNET_OK;
     void* p = nullptr;
     if (cudaMalloc(&p, 3 * 1024 * sizeof(uint2)) != cudaSuccess) {
@@ -48,7 +48,7 @@ sevennet_status radial_pack(sevennet_model* M, LayerDev& L) {
     }
     M->allocations.push_back(p);
     L.mlp1F = static_cast<uint2*>(p);
-    radial_pack_kernel<<<8, 128>>>(L.mlp1T, L.mlp1F);
+    radial_pack_kernel<<<8, 128>>>(W2T, L.mlp1F);
     SN_CUDA(cudaGetLastError());
     return SEVENNET_OK;
 }

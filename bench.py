@@ -57,28 +57,42 @@ def block_paths(spec, t):
     return out
 
 
-def conv_flops_per_edge(spec, t, adjoint, tensor_core):
-    """Algorithmic FLOPs of the fused convolution kernel per edge for block t,
-    split into (FFMA work, tensor-core work).  With tensor_core, the MLP matrix
-    products with H-wide inputs (H x H and H x W) run on tensor cores.  The
-    adjoint of an evaluation runs over unordered pairs of edges: the radial MLP
-    (recompute and input gradient) and the G matrices once per pair, the tensor
-    product once per direction, so per edge the former count half."""
+def conv_flops_per_edge(spec, t, adjoint, fp32):
+    """Algorithmic FLOPs of the convolution of block t per edge in an evaluation, split
+    into (FP32 lanes, tensor cores).  The matrix products with H-wide inputs (H x H and
+    H x W) run on tensor cores, in FP32 as six BF16 products of three-term operands.
+
+    Adjoint, over unordered pairs of edges: the radial MLP (recompute and input
+    gradient) and the G matrices once per pair, so half per edge; per direction and
+    channel t = G g, dE/dw = x t, dE/dx = w t; dE/dY (of the paths with l2 > 0) by the
+    cheaper of two forms: the coupling per direction, or S = w x g per direction and the
+    coupling once per pair.
+
+    Forward with a 64-wide radial MLP: the sums over edges of w x Y (a scalar product
+    contracts x with Y first), the hidden layers once per pair; the coupling, once per
+    receiver, is left out.  Forward with a 32-wide one: G per edge, t = G x, times w."""
     H, NB = spec.mlp_hidden, spec.n_basis
     paths = block_paths(spec, t)
     W = sum(p[3] for p in paths)
-    first = 2 * NB * H                                         # basis -> hidden, FFMA always
+    first = 2 * NB * H                                         # basis -> hidden
     mm = 2 * (H * H + H * W)                                   # hidden -> hidden -> W
     g = sum(2 * CG_NNZ[p[:3]] for p in paths)                 # G matrices
-    if not adjoint:
-        tp = sum(2 * mu * ((2 * l1 + 1) * (2 * l3 + 1) + (2 * l3 + 1)) for l1, l2, l3, mu in paths)
-        mlp_alu, mlp_tc = (first, mm) if tensor_core else (first + mm, 0)
-        return mlp_alu + g + tp, mlp_tc
-    tp = sum(2 * mu * ((2 * l1 + 1) * (2 * l3 + 1) + 2 * (2 * l1 + 1) + CG_NNZ[(l1, l2, l3)])
-             for l1, l2, l3, mu in paths)
-    # forward recompute + input gradient of the MLP, and the G matrices, once per pair
-    mlp_alu, mlp_tc = (first, mm) if tensor_core else (first + mm, 0)
-    return mlp_alu + g // 2 + tp, mlp_tc
+    products = 6 if fp32 else 1
+    if adjoint:
+        tp = 0
+        for l1, l2, l3, mu in paths:
+            n13, nnz = (2 * l1 + 1) * (2 * l3 + 1), CG_NNZ[(l1, l2, l3)]
+            tp += mu * (2 * n13 + 4 * (2 * l1 + 1) + (min(2 * nnz, 2 * n13 + nnz) if l2 else 0))
+        # recompute and input gradient of the MLP: twice half a pair's
+        return first + g // 2 + tp, products * mm
+    if H == 64:
+        tp = 0
+        for l1, l2, l3, mu in paths:
+            n1, n2 = 2 * l1 + 1, 2 * l2 + 1
+            tp += 2 * mu * (n1 if l2 == 0 else 1 + n2 if l1 == 0 else n1 + 1 if l3 == 0 else n1 * (1 + n2))
+        return first // 2 + tp, products * 2 * (H * H // 2 + H * W)
+    tp = sum(2 * mu * ((2 * l1 + 1) * (2 * l3 + 1) + (2 * l3 + 1)) for l1, l2, l3, mu in paths)
+    return first + g + tp, products * mm
 
 
 def fp32_alu_peak_tflops(n_sm, clock_mhz):
@@ -586,27 +600,26 @@ def main():
     # roofline of the dominant kernel family (the convolution adjoint)
     fam = max(("conv_bwd", "conv_fwd"), key=lambda k: prof.get(k, (0, 0))[0])
     tot_ms, n_launch = prof[fam]
-    tc = args.precision == "bf16"
-    per = [conv_flops_per_edge(spec, t, fam == "conv_bwd", tc) for t in range(spec.n_layers)]
+    bf16 = args.precision == "bf16"
+    per = [conv_flops_per_edge(spec, t, fam == "conv_bwd", not bf16) for t in range(spec.n_layers)]
     alu_step = sum(a for a, _ in per) * n_edges
     tc_step = sum(b for _, b in per) * n_edges
     achieved = alu_step * args.steps / (tot_ms / 1e3) / 1e12
     alu = measure_alu_peak(sn, local)
     peak = alu["peak_tflops"]
     roofline = {"bound": "alu", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
-                "traffic": traffic_for(fam) if args.workload == WORKLOAD and tc else None,
+                "traffic": traffic_for(fam) if args.workload == WORKLOAD and bf16 else None,
                 "kernel": fam, "share_of_step": tot_ms / dev_ms,
                 "peak_source": "measured FP32 FMA throughput (of measured; sevennet_fp32_peak, best of the "
                                "scalar and packed forms)", "alu_peak": alu,
                 "peak_from_unit_counts": fp32_alu_peak_tflops(n_sm, 2070.0),
                 "alu_flops_per_step": alu_step}
-    if tc:
-        peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))) if os.path.exists(
-            os.path.join(ROOT, "MEASURED_PEAKS.json")) else {"bf16_tflops": 1900.0}
-        t_ach = tc_step * args.steps / (tot_ms / 1e3) / 1e12
-        roofline["tensor"] = {"achieved": t_ach, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
-                              "frac": t_ach / peaks["bf16_tflops"], "flops_per_step": tc_step,
-                              "peak_source": "MEASURED_PEAKS.json bf16_tflops (of measured)"}
+    peaks = json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json"))) if os.path.exists(
+        os.path.join(ROOT, "MEASURED_PEAKS.json")) else {"bf16_tflops": 1900.0}
+    t_ach = tc_step * args.steps / (tot_ms / 1e3) / 1e12
+    roofline["tensor"] = {"achieved": t_ach, "peak": peaks["bf16_tflops"], "unit": "TFLOP/s",
+                          "frac": t_ach / peaks["bf16_tflops"], "flops_per_step": tc_step,
+                          "peak_source": "MEASURED_PEAKS.json bf16_tflops (of measured)"}
 
     line = {"metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
             "warmup": args.warmup, "ms_per_step": ms_per_step, "median_ms_per_step": med_ms,

@@ -286,7 +286,7 @@ static sevennet_status dev_upload(sevennet_model* M, const std::vector<T>& h, T*
     return SEVENNET_OK;
 }
 
-// Gives a device array back before the model is destroyed (waits for the work that reads it).
+// Gives a device array back before the model is destroyed.
 template <typename T>
 static void dev_release(sevennet_model* M, T* p) {
     M->allocations.erase(std::remove(M->allocations.begin(), M->allocations.end(), (void*)p), M->allocations.end());
@@ -886,6 +886,7 @@ sevennet_status sevennet_create_model(const sevennet_model_config* cfg, const do
     }
     const int H = cfg->mlp_hidden, NB = cfg->n_basis;
     M->layers.resize(M->T);
+    std::vector<float*> temps;               // radial-MLP weights in FP32, until their BF16 terms and fragments are made
     for (int t = 0; t < M->T; ++t) {
         LayerDev& L = M->layers[t];
         std::vector<PathH> paths;
@@ -1044,6 +1045,7 @@ sevennet_status sevennet_create_model(const sevennet_model_config* cfg, const do
         set_error("weight preparation failed: %s", cudaGetErrorString(cudaGetLastError()));
         return fail(SEVENNET_ECUDA);
     }
+    for (float* p : temps) dev_release(M, p);
     if (cudaStreamCreateWithFlags(&M->stream, cudaStreamNonBlocking) != cudaSuccess) {
         cudaGetLastError();
         set_error("cudaStreamCreate failed");

@@ -15,7 +15,7 @@
 // Forward: one CTA owns a contiguous range of receivers (balanced by edge
 // count) and walks its edges, sorted by receiver, in chunks of EC edges.
 // Adjoint: one CTA per tile of up to 4 chunks, tiles in edge order.  Per chunk:
-//   A  geometry: r, unit vector, Y (l <= 2), Bessel basis x envelope  (FP32)
+//   A  geometry: r, unit vector, Y (l <= 3), Bessel basis x envelope  (FP32)
 //   B  radial MLP hidden layers
 //   C  G matrices of every path for every edge of the chunk
 //   D  w = H2 @ W3 for all W columns into shared memory   (tensor cores)

@@ -1,5 +1,5 @@
-// Forward tensor-product convolution of one interaction block on the tensor
-// cores (BF16 path): Eq. 3 with the uvu product of Figure 2b.
+// Chunked forward tensor-product convolution of one interaction block on the tensor
+// cores (BF16 path of the calls that do not stream): Eq. 3 with the uvu product of Figure 2b.
 //
 // For path p = (l1, l2, l3), channel u and receiver v,
 //   m_v[p][m3, u] = sum_{e into v} sum_{m1} (w_e[p, u] x_src(e)[l1][m1, u]) G_e^p[m1, m3],

@@ -528,11 +528,11 @@ sevennet_status run_model(sevennet_model* M, Workspace* ws, const BatchHost& b, 
 // refresh, [1] two atoms closer than 1e-8 A, [2] reverse edge missing, [3]
 // species out of range, [FLAG_GX_OVERFLOW], [FLAG_EDGE_OVERFLOW] edges beyond
 // the capacity, [FLAG_EDGE_NEED] the largest edge count asked for,
-// [FLAG_COPY_TIMEOUT] a bulk copy not completed within its bounded wait.
+// [FLAG_COPY_TIMEOUT] a bounded wait of a forward convolution ran out.
 constexpr int FLAG_WORDS = 8;
 constexpr int FLAG_EDGE_OVERFLOW = 4;
 constexpr int FLAG_EDGE_NEED = 6;
-constexpr int FLAG_COPY_TIMEOUT = 7;     // a bounded wait for a bulk copy ran out
+constexpr int FLAG_COPY_TIMEOUT = 7;
 
 // Deterministic scatter of dE/dx in the convolution adjoint: every per-edge
 // contribution v is added as the 64-bit integer round(v * 2^36) (fixed point),
@@ -545,7 +545,7 @@ constexpr long long GX_SENTINEL = 1LL << 57;
 constexpr int FLAG_GX_OVERFLOW = 5;
 
 // kernels launchers (conv.cu / node.cu)
-// flags (may be null) receives FLAG_COPY_TIMEOUT from the tensor-core forward
+// flags (may be null) receives FLAG_COPY_TIMEOUT from the chunked tensor-core forward
 void launch_conv_fwd(const LayerDev& L, int H, sevennet_precision prec, int64_t n_atoms,
                      int64_t n_edges, const int* row_ptr, const int* dst, const int* src,
                      const float4* geom, const float* x, float* m, cudaStream_t st, int* flags = nullptr);
@@ -558,7 +558,7 @@ void launch_conv_bwd(const LayerDev& L, int H, sevennet_precision prec, int64_t 
                      const float4* geom, const float* x, const float* gm, float* gx,
                      unsigned long long* gxq, int* flags, float* gd, cudaStream_t st);
 sevennet_status conv_configure(int H, const std::vector<LayerDev>& layers);
-// tensor-core forward of the BF16 path (conv_fwd_tc.cu)
+// chunked tensor-core forward of the BF16 path (conv_fwd_tc.cu)
 size_t conv_tc_smem_bytes(const ConvDesc& D, int H);
 sevennet_status conv_configure_fwd_tc(int H, size_t need);
 void launch_conv_fwd_tc(const LayerDev& L, int H, int64_t n_atoms, int64_t n_edges, const int* row_ptr,

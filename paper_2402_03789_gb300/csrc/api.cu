@@ -505,7 +505,8 @@ int ws_h2_bytes(const sevennet_model* M, const Workspace* ws) { return std::min(
 // Grows the workspace to the given sizes (the server's bytes_per_atom counts what an atom
 // takes here).  Nothing happens (and nothing waits)
 // when the capacities suffice; a reallocation frees the old buffer first, and
-// cudaFree waits for the work that may still use it.
+// cudaFree waits for the work that may still use it.  A capacity is 0 while its buffers
+// are replaced, so that after a failed call the next one allocates them again.
 sevennet_status ws_reserve(sevennet_model* M, Workspace* ws, int64_t n_atoms, int64_t n_edges,
                            int64_t n_bins, int64_t n_structs, cudaStream_t st) {
     (void)st;
@@ -517,6 +518,7 @@ sevennet_status ws_reserve(sevennet_model* M, Workspace* ws, int64_t n_atoms, in
     }
     if (n_atoms > ws->cap_atoms) {
         const int64_t N = std::max<int64_t>(n_atoms, 16);
+        ws->cap_atoms = 0;
         const int T = M->T;
         SN_TRY(ws_alloc(ws, &ws->bin_of, N));
         SN_TRY(ws_alloc(ws, &ws->perm, N));
@@ -541,6 +543,7 @@ sevennet_status ws_reserve(sevennet_model* M, Workspace* ws, int64_t n_atoms, in
     if (n_edges > ws->cap_edges) {
         const int64_t E = std::max<int64_t>(n_edges, 1024);
         SN_CHECK(E < (1LL << 31) - 1, SEVENNET_EOVERFLOW, "edge count exceeds 2^31");
+        ws->cap_edges = 0;
         SN_TRY(ws_alloc(ws, &ws->dst, E));
         SN_TRY(ws_alloc(ws, &ws->src, E));
         SN_TRY(ws_alloc(ws, &ws->shift, E * 3));
@@ -574,6 +577,7 @@ sevennet_status ws_reserve(sevennet_model* M, Workspace* ws, int64_t n_atoms, in
     }
     if (n_bins + 1 > ws->cap_bins) {
         const int64_t B = std::max<int64_t>(n_bins + 1, 64);
+        ws->cap_bins = 0;
         SN_TRY(ws_alloc(ws, &ws->bin_count, B + 1));
         SN_TRY(ws_alloc(ws, &ws->bin_start, B + 1));
         SN_TRY(ws_alloc(ws, &ws->bin_fill, B + 1));
@@ -581,6 +585,7 @@ sevennet_status ws_reserve(sevennet_model* M, Workspace* ws, int64_t n_atoms, in
     }
     if (n_structs > ws->cap_structs) {
         const int64_t S = std::max<int64_t>(n_structs, 4);
+        ws->cap_structs = 0;
         SN_TRY(ws_alloc(ws, &ws->cells, S * 9));
         SN_TRY(ws_alloc(ws, &ws->inv_cells, S * 9));
         SN_TRY(ws_alloc(ws, &ws->sdesc, S * 16));

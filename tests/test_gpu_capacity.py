@@ -74,3 +74,31 @@ def test_server_memory_stays_within_its_budget(prec):
     srv.close()
     model.close()
     assert 0.97 * budget <= used <= budget + slots * 45 * (2 << 20)
+
+
+def test_call_after_one_that_ran_out_of_memory():
+    """24,000 atoms with 600 MB of device memory left (they need 1.2 GB) end with ENOMEM
+    half way through the workspace; a small call after that allocates again what the
+    failed one had given back, and gives the bits of before."""
+    import torch
+    import paper_2402_03789_gb300 as sn
+    spec = MODEL_SEVENNET0
+    model = sn.SevenNet(spec, normal_weights(oracle.n_params(spec)))
+    s = random_structure({"Si": 64, "O": 128}, 2.2, 1.6, seed=5)
+    before = model.evaluate(s.pos, s.cell, s.species, "fp32")
+    rng = np.random.default_rng(0)
+    k = 29                                        # a lattice of 24,389 sites, 2.6 A apart
+    pos = np.stack(np.meshgrid(*[np.arange(k)] * 3, indexing="ij"), -1).reshape(-1, 3) * 2.6
+    species = rng.integers(0, 3, len(pos)).astype(np.int32)
+    torch.cuda.empty_cache()
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - (600 << 20), dtype=torch.uint8, device="cuda")
+    try:
+        with pytest.raises(sn.SevenNetError) as err:
+            model.evaluate(pos, np.eye(3) * (2.6 * k), species, "fp32")
+        assert err.value.status == -2
+        after = model.evaluate(s.pos, s.cell, s.species, "fp32")
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    assert after[0] == before[0] and np.array_equal(after[1], before[1]) and np.array_equal(after[2], before[2])
+    model.close()

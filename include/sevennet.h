@@ -193,7 +193,9 @@ sevennet_status sevennet_eval_energy_forces_virial(sevennet_model* model, int64_
  * radial MLP, rows of gradients below 4,096 bytes an atom, such as 32x0e+32x1e, or
  * blocks whose channels do not fit the streaming kernel's shared memory) group a
  * receiver's edges from chunk boundaries that move with the batch; there the
- * results agree to FP32 rounding carried through the BF16 operands. */
+ * results agree to FP32 rounding carried through the BF16 operands.  A model that
+ * streams keeps the chunked forward from the first call on whose lists leave too
+ * little device memory for the streaming one's activations (128 or 256 bytes a pair). */
 sevennet_status sevennet_eval_batch_dev(sevennet_model* model, int32_t n_structs,
                                         const int64_t* atom_offsets, const double* cells,
                                         const int32_t* pbc, const int32_t* species_dev,

@@ -556,25 +556,6 @@ sevennet_status ws_reserve(sevennet_model* M, Workspace* ws, int64_t n_atoms, in
         SN_TRY(ws_alloc(ws, &ws->gd, E * 3));
         ws->cap_edges = E;
     }
-    const int64_t grad = std::max<int64_t>(ws->cap_atoms * st_grad_bytes(M), (ws->cap_edges + 1) / 2 * ws_h2_bytes(M, ws));
-    if (grad > ws->grad_bytes) {
-        ws->grad_bytes = 0;
-        SN_TRY(ws_alloc(ws, &ws->grad, grad));
-        ws->grad_bytes = grad;
-    }
-    if (M->h2_bytes && ws->cap_edges / 4 + ws->cap_atoms > ws->cap_quads) {
-        ws->cap_quads = 0;
-        SN_TRY(ws_alloc(ws, &ws->quads, ws->cap_edges / 4 + ws->cap_atoms));
-        ws->cap_quads = ws->cap_edges / 4 + ws->cap_atoms;
-    }
-    {
-        const int64_t N = ws->cap_atoms;
-        ws->gxq = reinterpret_cast<unsigned long long*>(ws->grad);
-        ws->gx = reinterpret_cast<float*>(ws->gxq + N * M->x_max);
-        ws->gy = ws->gx + N * M->x_max;
-        ws->gh = ws->gy + N * M->y_max;
-        ws->h = ws->gh + N * M->h_max;
-    }
     if (n_bins + 1 > ws->cap_bins) {
         const int64_t B = std::max<int64_t>(n_bins + 1, 64);
         ws->cap_bins = 0;
@@ -598,6 +579,35 @@ sevennet_status ws_reserve(sevennet_model* M, Workspace* ws, int64_t n_atoms, in
         SN_TRY(ws_alloc(ws, &ws->partial, partials * 10));
         ws->cap_partial = partials;
     }
+    // Last, the gradient block with the pairs' hidden activations and the groups of four.  Where
+    // they do not fit, dense lists near the device's memory, the block holds the gradients alone
+    // and the workspace's evaluations keep the chunked forward.
+    const int64_t grads = ws->cap_atoms * st_grad_bytes(M), pairs = (ws->cap_edges + 1) / 2;
+    const int64_t quads = ws->cap_edges / 4 + ws->cap_atoms;
+    if (ws_h2_bytes(M, ws)) {
+        if (quads > ws->cap_quads) {
+            ws->cap_quads = 0;
+            if (ws_alloc(ws, &ws->quads, quads) == SEVENNET_OK) ws->cap_quads = quads;
+            else ws->h2_max = 0;
+        }
+        const int64_t grad = std::max<int64_t>(grads, pairs * ws_h2_bytes(M, ws));
+        if (grad > ws->grad_bytes) {
+            ws->grad_bytes = 0;
+            if (ws_alloc(ws, &ws->grad, grad) == SEVENNET_OK) ws->grad_bytes = grad;
+            else ws->h2_max = 0;
+        }
+    }
+    if (grads > ws->grad_bytes) {
+        ws->grad_bytes = 0;
+        SN_TRY(ws_alloc(ws, &ws->grad, grads));
+        ws->grad_bytes = grads;
+    }
+    const int64_t N = ws->cap_atoms;
+    ws->gxq = reinterpret_cast<unsigned long long*>(ws->grad);
+    ws->gx = reinterpret_cast<float*>(ws->gxq + N * M->x_max);
+    ws->gy = ws->gx + N * M->x_max;
+    ws->gh = ws->gy + N * M->y_max;
+    ws->h = ws->gh + N * M->h_max;
     return SEVENNET_OK;
 }
 
@@ -753,12 +763,13 @@ sevennet_status run_model(sevennet_model* M, Workspace* ws, const BatchHost& b, 
     // the memory of dE/dd, which the adjoint clears)
     prof_begin(&M->prof, PF_NEIGHBORS, st, &ev);
     build_pairs(ws, N, st);
-    if (M->h2_bytes) {
+    const bool h2 = ws_h2_bytes(M, ws) > 0;
+    if (h2) {
         launch_pair_of((ws->cap_edges + 1) / 2, N, ws->row_ptr, ws->rev, ws->pair_ptr, ws->p_e,
                        reinterpret_cast<int*>(ws->gd), st);
         launch_quads(N, ws->row_ptr, ws->quad_ptr, ws->quads, st);
     }
-    const int n_pre = M->h2_bytes ? 5 : 3;
+    const int n_pre = h2 ? 5 : 3;
     prof_end(&M->prof, PF_NEIGHBORS, st, ev, n_pre);
     count_launches(n_pre);
     model_embed(M, ws, N, st);

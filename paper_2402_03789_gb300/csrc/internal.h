@@ -453,7 +453,7 @@ struct Workspace {
     // the pairs' hidden activations there while a convolution runs (all five are dead then)
     unsigned char* grad = nullptr;
     int64_t grad_bytes = 0;
-    int h2_max = 256;             // room for hidden activations per pair (128: BF16 evaluations only)
+    int h2_max = 256;             // room for hidden activations per pair (128: BF16 evaluations only; 0: they did not fit)
     float* h = nullptr;           // [N][h_max]
     float* xs = nullptr;          // [T][N][x_max]
     float* ys = nullptr;          // [T][N][y_max]

@@ -102,3 +102,42 @@ def test_call_after_one_that_ran_out_of_memory():
         torch.cuda.empty_cache()
     assert after[0] == before[0] and np.array_equal(after[1], before[1]) and np.array_equal(after[2], before[2])
     model.close()
+
+
+def test_hidden_activations_that_do_not_fit_leave_the_chunked_forward():
+    """A list of some 100 edges an atom, where the pairs' FP32 hidden activations (129 edges of
+    room: 16.5 KB an atom) are larger than the gradients whose memory they share (7.2 KB):
+    with memory for the gradients alone the call still runs, in the chunked kernels."""
+    import dataclasses
+    import torch
+    import paper_2402_03789_gb300 as sn
+    spec = dataclasses.replace(benchmark_model(3, 32, 2), r_cut=7.0)
+    w = normal_weights(oracle.n_params(spec))
+    rng = np.random.default_rng(3)
+    k = 28
+    grid = np.stack(np.meshgrid(*[np.arange(k)] * 3, indexing="ij"), -1).reshape(-1, 3)
+    pos, cell = (grid + rng.uniform(-0.16, 0.16, grid.shape)) * 2.4, np.eye(3) * (2.4 * k)
+    species = rng.integers(0, 3, len(pos)).astype(np.int32)
+    torch.cuda.empty_cache()
+
+    def run():
+        model = sn.SevenNet(spec, w)
+        first = model.lib.sevennet_launch_count()
+        out = model.evaluate(pos, cell, species, "fp32")
+        return model, out, model.lib.sevennet_launch_count() - first
+
+    free = torch.cuda.mem_get_info()[0]
+    model, (E1, F1, W1), n1 = run()
+    used = free - torch.cuda.mem_get_info()[0]
+    model.close()
+    short = len(pos) * (16500 - 7200) // 2
+    filler = torch.empty(torch.cuda.mem_get_info()[0] - used + short, dtype=torch.uint8, device="cuda")
+    try:
+        model, (E2, F2, W2), n2 = run()
+        model.close()
+    finally:
+        del filler
+        torch.cuda.empty_cache()
+    assert n2 < n1                                # no hidden layers once per pair, no groups of four
+    e_pa, f_rel, w_rel = errors(E2, F2, W2, E1, F1, W1, len(pos))
+    assert e_pa <= 1e-6 and f_rel <= 1e-5 and w_rel <= 1e-5
